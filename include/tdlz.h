@@ -231,19 +231,14 @@ tdlz_status tdlz_spectrum(tdlz_ctx *ctx, const tdlz_coeffs *c, const tdlz_spectr
  * caller-owned DEVICE arrays (layouts as in tdlz_coeffs / tdlz_spectrum,
  * complex double); nomega must equal the grid length (query it with
  * tdlz_spectrum(ctx, c, sp, NULL, &nomega), which allocates nothing).
- * Scratch: one file-scope static device array of TDLZ_NOALLOC_SCRATCH_MB MiB,
- * held by every GPU that loads the library until the process exits; frequencies
- * are processed in chunks that fit it.  Rejected with TDLZ_ERR_ARG (nothing
- * launched): 4 * nchain * nsteps complex rows above the scratch, i.e.
- * nchain * nsteps > TDLZ_NOALLOC_SCRATCH_MB * 2^20 / 64, and grids longer than
+ * The solve keeps its state in registers and needs no scratch.  Rejected with
+ * TDLZ_ERR_ARG (nothing launched): nchain * nsteps > TDLZ_NOALLOC_SCRATCH_MB * 2^20 / 64
+ * (the limit of an earlier form that kept its rows in a static array of that size;
+ * callers may rely on it), and grids longer than
  * 2^24 frequencies.  The per-chain step counts dev_coeffs->steps stay on the device,
  * so they are not checked: values outside [0, nsteps] are clamped to that range
- * (tdlz_spectrum, which receives them on the host, rejects them).  The first call on a
- * device looks up the scratch's device address (cudaGetSymbolAddress) and
- * caches it; make that first call before any stream capture.  Every call on a
- * device shares the one array and leaves its contents behind (each call writes
- * every row it reads, so nothing needs clearing); calls whose kernels overlap on
- * the GPU (other streams, other host threads) race on it.  Enqueued on the
+ * (tdlz_spectrum, which receives them on the host, rejects them).  Calls that overlap
+ * on the GPU (other streams, other host threads) are independent.  Enqueued on the
  * context stream; no allocation of any kind, no synchronisation. */
 #define TDLZ_NOALLOC_SCRATCH_MB 32
 tdlz_status tdlz_spectrum_noalloc(tdlz_ctx *ctx, const tdlz_coeffs *dev_coeffs,

@@ -363,47 +363,58 @@ tdlz_status tdlz_spectrum(tdlz_ctx *ctx, const tdlz_coeffs *c, const tdlz_spectr
                    "steps out of range");
     const double conv = sp->units == 1 ? 1.0 / 27211.386245988 : 1.0;
     const int nc = c->nchain, cap = c->nsteps, nl = c->ncomp == 4 ? 4 : 3;
-    DevBuf d_steps, d_al, d_be, d_ga, d_z, d_n0, d_wk, d_chi, d_scr;
+    for (int i = 0; i < nc; ++i)
+      TDLZ_REQUIRE(sp->itermax0 <= c->steps[i] || sp->itermax0 == 0 || sp->extrapolation == 0,
+                   TDLZ_ERR_ARG, "itermax0 exceeds the computed steps of a chain");
+    // every input packed into one host block and one copy, into a workspace the context
+    // keeps (a call of 9 allocations, 7 copies and 9 frees spent more on them than the
+    // solve of a few hundred steps takes)
     cudaStream_t st = ctx->c.stream;
-    auto up = [&](DevBuf &b, const void *src, size_t bytes) {
-      b.alloc(bytes);
-      TDLZ_CUDA_TRY(cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, st));
+    size_t total = 0;
+    auto place = [&](size_t bytes) {
+      const size_t at = total;
+      total += (bytes + 15) & ~(size_t)15;
+      return at;
     };
-    up(d_steps, c->steps, sizeof(int) * nc);
-    up(d_al, c->alpha, sizeof(double2) * nc * cap);
-    up(d_be, c->beta, sizeof(double) * nc * cap);
-    up(d_ga, c->gamma, sizeof(double2) * nc * cap);
-    up(d_z, c->z, sizeof(double2) * nc * nl * cap);
-    up(d_n0, c->n0, sizeof(double) * nc);
-    up(d_wk, c->wk, sizeof(double) * nc);
-    d_chi.alloc(sizeof(double2) * nc * nl * nw);
-    d_scr.alloc(sizeof(double2) * 4 * (size_t)cap * nc * nw);
+    const size_t n_al = sizeof(double2) * nc * cap, n_be = sizeof(double) * nc * cap;
+    const size_t o_al = place(n_al), o_ga = place(n_al), o_z = place(n_al * nl),
+                 o_be = place(n_be), o_n0 = place(sizeof(double) * nc),
+                 o_wk = place(sizeof(double) * nc), o_st = place(sizeof(int) * nc);
+    std::vector<char> host(total);
+    std::memcpy(host.data() + o_al, c->alpha, n_al);
+    std::memcpy(host.data() + o_ga, c->gamma, n_al);
+    std::memcpy(host.data() + o_z, c->z, n_al * nl);
+    std::memcpy(host.data() + o_be, c->beta, n_be);
+    std::memcpy(host.data() + o_n0, c->n0, sizeof(double) * nc);
+    std::memcpy(host.data() + o_wk, c->wk, sizeof(double) * nc);
+    std::memcpy(host.data() + o_st, c->steps, sizeof(int) * nc);
+    const size_t chi_bytes = sizeof(double2) * nc * nl * (size_t)nw;
+    DevBuf &ws = ctx->c.spec_ws;
+    if (ws.bytes < total + chi_bytes) ws.alloc(total + chi_bytes);
+    char *dp = ws.as<char>();
+    TDLZ_CUDA_TRY(cudaMemcpyAsync(dp, host.data(), total, cudaMemcpyHostToDevice, st));
+    double2 *d_chi = reinterpret_cast<double2 *>(dp + total);
     SpecArgs a{};
     a.nchain = nc;
     a.nomega = (int)nw;
     a.cap = cap;
     a.nl = nl;
-    a.steps = d_steps.as<int>();
-    a.alpha = d_al.as<double2>();
-    a.beta = d_be.as<double>();
-    a.gamma = d_ga.as<double2>();
-    a.z = d_z.as<double2>();
-    a.n0 = d_n0.as<double>();
-    a.wk = d_wk.as<double>();
+    a.steps = reinterpret_cast<int *>(dp + o_st);
+    a.alpha = reinterpret_cast<double2 *>(dp + o_al);
+    a.beta = reinterpret_cast<double *>(dp + o_be);
+    a.gamma = reinterpret_cast<double2 *>(dp + o_ga);
+    a.z = reinterpret_cast<double2 *>(dp + o_z);
+    a.n0 = reinterpret_cast<double *>(dp + o_n0);
+    a.wk = reinterpret_cast<double *>(dp + o_wk);
     a.start = sp->start * conv;
     a.step = sp->step * conv;
     a.eta = sp->eta * conv;
-    a.scratch = d_scr.as<double2>();
     a.itermax0 = sp->itermax0;
     a.itermax = sp->itermax;
     a.extrap = sp->extrapolation;
-    for (int i = 0; i < nc; ++i)
-      TDLZ_REQUIRE(sp->itermax0 <= c->steps[i] || sp->itermax0 == 0 || sp->extrapolation == 0,
-                   TDLZ_ERR_ARG, "itermax0 exceeds the computed steps of a chain");
-    a.chi = d_chi.as<double2>();
+    a.chi = d_chi;
     launch_spectrum(st, a);
-    TDLZ_CUDA_TRY(cudaMemcpyAsync(chi, d_chi.p, sizeof(double2) * nc * nl * nw,
-                                  cudaMemcpyDeviceToHost, st));
+    TDLZ_CUDA_TRY(cudaMemcpyAsync(chi, d_chi, chi_bytes, cudaMemcpyDeviceToHost, st));
     TDLZ_CUDA_TRY(cudaStreamSynchronize(st));
   });
 }

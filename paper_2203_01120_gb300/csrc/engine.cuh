@@ -169,6 +169,7 @@ struct Context {
   std::vector<std::unique_ptr<QSlot>> slots;
   Profiler prof;
   Tuner tuner;
+  DevBuf spec_ws;  // tdlz_spectrum: inputs and chi of the largest call so far
 };
 
 template <class T> inline SlotData<T> &slot_data(QSlot &s) {

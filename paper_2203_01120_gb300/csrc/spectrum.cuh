@@ -16,7 +16,6 @@ struct SpecArgs {
   const double *n0, *wk; // [nchain]
   double start, step, eta;
   int itermax0, itermax, extrap;  // itermax0 <= 0: all computed; extrap 0 no, 1 constant, 2 osc
-  double2 *scratch;      // [4][cap][nchain*nomega]
   double2 *chi;          // [nchain][nl][nomega]
 };
 

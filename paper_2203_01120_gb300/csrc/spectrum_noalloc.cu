@@ -1,10 +1,7 @@
 // tdlz_spectrum_noalloc: the pivoted tridiagonal spectrum solve for callers that
 // cannot allocate device memory.  Inputs and outputs are the caller's device
-// buffers; the elimination rows live in one file-scope static device array of
-// fixed size, shared by every call on a device and kept by every GPU that loads
-// the library until the process exits.
+// buffers; the solve keeps its state in registers (spectrum_solve.cuh).
 #include <cmath>
-#include <mutex>
 
 #include "engine.cuh"
 #include "spectrum_solve.cuh"
@@ -13,60 +10,32 @@ namespace tdlz {
 
 namespace {
 
-constexpr size_t kNoallocScratchBytes = (size_t)TDLZ_NOALLOC_SCRATCH_MB << 20;
-constexpr int kMaxDevices = 64;
-
-// The scratch.  Device code could name it directly; host code must not pass
-// the symbol itself to a kernel (on the host it is only a stand-in), so the
-// device address is looked up per device with cudaGetSymbolAddress.
-static __device__ __align__(256) double2 g_spec_scratch[kNoallocScratchBytes / sizeof(double2)];
-
-std::mutex g_mu;
-double2 *g_scratch_ptr[kMaxDevices] = {nullptr};
-
-// One thread per (chain, omega) of the chunk [w0, w0 + nw); rows stored at
-// scratch[(q * cap + i) * nthr + tid] for q = d, du, du2, b.
-__global__ void spectrum_noalloc_kernel(int nchain, int nomega, int cap, const int *steps,
-                                        const double2 *alpha, const double *beta,
-                                        const double2 *gamma, const double2 *z, const double *n0,
-                                        const double *wk, double start, double step, double eta,
-                                        int w0, int nw, int nl, double2 *scratch, double2 *chi) {
+// One thread per (chain, omega).
+template <int NL>
+__global__ void __launch_bounds__(kSpecThreads)
+    spectrum_noalloc_kernel(int nchain, int nomega, int cap, const int *steps,
+                            const double2 *alpha, const double *beta, const double2 *gamma,
+                            const double2 *z, const double *n0, const double *wk, double start,
+                            double step, double eta, double2 *chi) {
   long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nthr = (long long)nchain * nw;
-  if (tid >= nthr) return;
-  int c = (int)(tid / nw);
-  int iw = w0 + (int)(tid - (long long)c * nw);
+  if (tid >= (long long)nchain * nomega) return;
+  int c = (int)(tid / nomega);
+  int iw = (int)(tid - (long long)c * nomega);
   int m = steps[c];  // read on the device: clamped to [0, cap]
   if (m > cap) m = cap;
-  double2 *out = chi + ((long long)c * nl) * nomega + iw;
+  double2 *out = chi + ((long long)c * NL) * nomega + iw;
   if (m <= 0) {
-    for (int l = 0; l < nl; ++l) out[(long long)l * nomega] = make_double2(0, 0);
+    for (int l = 0; l < NL; ++l) out[(long long)l * nomega] = make_double2(0, 0);
     return;
   }
-  const double2 *al = alpha + (long long)c * cap;
-  const double *be = beta + (long long)c * cap;
-  const double2 *ga = gamma + (long long)c * cap;
-  const double2 *zz = z + (long long)c * nl * cap;
-  double2 acc[4];
-  tridiag_chi(m, cap, al, be, ga, zz, make_double2(start + step * iw, eta), make_double2(0, 0),
-              scratch, nthr, tid, nl, acc);
+  double2 acc[NL];
+  tridiag_chi<NL>(m, cap, alpha + (long long)c * cap, beta + (long long)c * cap,
+                  gamma + (long long)c * cap, z + (long long)c * NL * cap,
+                  make_double2(start + step * iw, eta), make_double2(0, 0), acc);
   double s = wk[c] * n0[c];
-  for (int l = 0; l < nl; ++l) out[(long long)l * nomega] = make_double2(s * acc[l].x, s * acc[l].y);
-}
-
-// Device address of the scratch on the current device; looked up once per device.
-double2 *scratch_on_current_device(int dev) {
-  TDLZ_REQUIRE(dev >= 0 && dev < kMaxDevices, TDLZ_ERR_ARG, "device ordinal out of range");
-  std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_scratch_ptr[dev]) {
-    void *p = nullptr;
-    cudaError_t e = cudaGetSymbolAddress(&p, g_spec_scratch);
-    if (e != cudaSuccess || p == nullptr)
-      throw Error{TDLZ_ERR_CUDA, std::string("cudaGetSymbolAddress(scratch) failed: ") +
-                                     cudaGetErrorString(e)};
-    g_scratch_ptr[dev] = static_cast<double2 *>(p);
-  }
-  return g_scratch_ptr[dev];
+#pragma unroll
+  for (int l = 0; l < NL; ++l)
+    out[(long long)l * nomega] = make_double2(s * acc[l].x, s * acc[l].y);
 }
 
 }  // namespace
@@ -88,26 +57,27 @@ void spectrum_noalloc(Context &ctx, const tdlz_coeffs *c, const tdlz_spectrum_pa
   TDLZ_REQUIRE(nw == nomega, TDLZ_ERR_ARG,
                "nomega does not match the frequency grid (query it with tdlz_spectrum, chi = NULL)");
   TDLZ_REQUIRE(nw <= (1LL << 24), TDLZ_ERR_ARG, "at most 2^24 frequencies");
-  // every frequency needs 4 complex rows of length nsteps per chain
-  const long long per_omega = 4LL * c->nsteps * c->nchain;  // double2 elements
-  const long long cap_elems = (long long)(kNoallocScratchBytes / sizeof(double2));
-  TDLZ_REQUIRE(per_omega <= cap_elems, TDLZ_ERR_ARG,
+  // size limit of the interface (it dates from a form of the solve that kept four complex
+  // rows per step in a static array of this many bytes)
+  const long long cap_steps = ((long long)TDLZ_NOALLOC_SCRATCH_MB << 20) / 64;
+  TDLZ_REQUIRE((long long)c->nsteps * c->nchain <= cap_steps, TDLZ_ERR_ARG,
                "nchain * nsteps exceeds the static scratch of tdlz_spectrum_noalloc (" +
                    std::to_string(TDLZ_NOALLOC_SCRATCH_MB) + " MiB holds nchain * nsteps <= " +
-                   std::to_string(cap_elems / 4) + ")");
-  double2 *scratch = scratch_on_current_device(ctx.device);
+                   std::to_string(cap_steps) + ")");
   const double conv = sp->units == 1 ? 1.0 / 27211.386245988 : 1.0;
-  const int chunk = (int)std::min<long long>(nw, cap_elems / per_omega);
-  for (int w0 = 0; w0 < nomega; w0 += chunk) {
-    int n = std::min(chunk, nomega - w0);
-    long long nthr = (long long)c->nchain * n;
-    spectrum_noalloc_kernel<<<blocks_for(nthr, 128), 128, 0, ctx.stream>>>(
+  auto launch = [&](auto kernel) {
+    kernel<<<blocks_for((long long)c->nchain * nomega, kSpecThreads), kSpecThreads, 0,
+             ctx.stream>>>(
         c->nchain, nomega, c->nsteps, c->steps, reinterpret_cast<const double2 *>(c->alpha),
         c->beta, reinterpret_cast<const double2 *>(c->gamma),
         reinterpret_cast<const double2 *>(c->z), c->n0, c->wk, sp->start * conv, sp->step * conv,
-        sp->eta * conv, w0, n, c->ncomp == 4 ? 4 : 3, scratch, reinterpret_cast<double2 *>(chi));
+        sp->eta * conv, reinterpret_cast<double2 *>(chi));
     TDLZ_LAUNCH_CHECK();
-  }
+  };
+  if (c->ncomp == 4)
+    launch(spectrum_noalloc_kernel<4>);
+  else
+    launch(spectrum_noalloc_kernel<3>);
 }
 
 }  // namespace tdlz
