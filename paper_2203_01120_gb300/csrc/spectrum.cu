@@ -1,9 +1,8 @@
 // chi(omega) from the Lanczos tridiagonal matrix (Eqs.
 // resolvent_Liouvillian_Lanczos_q and post_processing), FP64 on the GPU.
 //
-// One thread per (chain, omega) solves (omega + i eta - T) x = e_1 by Gaussian
-// elimination with partial pivoting and forms chi_l = w n0 sum_i conj(z^l_i) x_i in the
-// same sweep (spectrum_solve.cuh).
+// One thread per (chain, omega, left vector l) solves (omega + i eta - T) x = e_1 and
+// forms chi_l = w n0 sum_i conj(z^l_i) x_i in the same sweep (spectrum_solve.cuh).
 #include <cmath>
 
 #include "spectrum.cuh"
@@ -16,12 +15,6 @@ namespace tdlz {
 struct Mob {
   double2 x[4];
 };
-
-__device__ __forceinline__ double pow2_scale(int mag) {
-  // 2^-e of the upper word of the largest component; 1 for zero and non-finite entries
-  const int e = (mag >> 20) - 1023;
-  return e > -1000 && e < 1000 ? __hiloint2double((1023 - e) << 20, 0) : 1.0;
-}
 
 __device__ __forceinline__ Mob mob_mul(const Mob &a, const Mob &b) {
   const double2 zero = make_double2(0.0, 0.0);
@@ -37,7 +30,7 @@ __device__ __forceinline__ Mob mob_mul(const Mob &a, const Mob &b) {
   int mag = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) mag = max(mag, spec_mag(r.x[i]));
-  const double sc = pow2_scale(mag);
+  const double sc = spec_pow2(mag);
 #pragma unroll
   for (int i = 0; i < 4; ++i) r.x[i] = make_double2(r.x[i].x * sc, r.x[i].y * sc);
   return r;
@@ -49,29 +42,29 @@ __device__ __forceinline__ void mob_apply(const Mob &a, double2 (&v)[2]) {
   double2 d0 = spec_mul(a.x[2], v[0]), d1 = spec_mul(a.x[3], v[1]);
   v[0] = make_double2(n0.x + n1.x, n0.y + n1.y);
   v[1] = make_double2(d0.x + d1.x, d0.y + d1.y);
-  const double sc = pow2_scale(max(spec_mag(v[0]), spec_mag(v[1])));
+  const double sc = spec_pow2(max(spec_mag(v[0]), spec_mag(v[1])));
 #pragma unroll
   for (int i = 0; i < 2; ++i) v[i] = make_double2(v[i].x * sc, v[i].y * sc);
 }
 
-template <int NL>
 __global__ void __launch_bounds__(kSpecThreads) spectrum_kernel(SpecArgs a) {
   long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nthr = (long long)a.nchain * a.nomega;
-  if (tid >= nthr) return;
-  int c = (int)(tid / a.nomega);
-  int iw = (int)(tid - (long long)c * a.nomega);
+  if (tid >= (long long)a.nchain * a.nomega * a.nl) return;
+  const long long ciw = tid / a.nl;
+  const int l = (int)(tid - ciw * a.nl);
+  const int c = (int)(ciw / a.nomega);
+  const int iw = (int)(ciw - (long long)c * a.nomega);
   int m = a.steps[c];
   if (a.itermax0 > 0 && a.itermax0 < m) m = a.itermax0;
-  double2 *out = a.chi + ((long long)c * NL) * a.nomega + iw;
+  double2 *out = a.chi + ((long long)c * a.nl + l) * a.nomega + iw;
   if (m <= 0) {
-    for (int l = 0; l < NL; ++l) out[(long long)l * a.nomega] = make_double2(0, 0);
+    *out = make_double2(0, 0);
     return;
   }
   const double2 *al = a.alpha + (long long)c * a.cap;
   const double *be = a.beta + (long long)c * a.cap;
   const double2 *ga = a.gamma + (long long)c * a.cap;
-  const double2 *zz = a.z + (long long)c * NL * a.cap;
+  const double2 *zz = a.z + ((long long)c * a.nl + l) * a.cap;
   double om = a.start + a.step * iw;
   double2 zw = make_double2(om, a.eta);
   // Extrapolated tail (Sec. 3.3): coefficients m..itermax-1 are the means of the
@@ -125,12 +118,9 @@ __global__ void __launch_bounds__(kSpecThreads) spectrum_kernel(SpecArgs a) {
     double2 bg = make_double2(be[m - 1] * ga[m - 1].x, be[m - 1] * ga[m - 1].y);
     tail = make_double2(bg.x * g.x - bg.y * g.y, bg.x * g.y + bg.y * g.x);
   }
-  double2 acc[NL];
-  tridiag_chi<NL>(m, a.cap, al, be, ga, zz, zw, tail, acc);
+  const double2 acc = tridiag_chi(m, al, be, ga, zz, zw, tail);
   double s = a.wk[c] * a.n0[c];
-#pragma unroll
-  for (int l = 0; l < NL; ++l)
-    out[(long long)l * a.nomega] = make_double2(s * acc[l].x, s * acc[l].y);
+  *out = make_double2(s * acc.x, s * acc.y);
 }
 
 // S(w) = -Im sum_ab P_ab chi_ba(w), chi[a][b][w] = chi_ba (chain a, row b)  (Eq. S_def)
@@ -151,12 +141,8 @@ void launch_structure_factor(cudaStream_t st, const double2 *chi, int nomega, co
 }
 
 void launch_spectrum(cudaStream_t st, const SpecArgs &a) {
-  long long nthr = (long long)a.nchain * a.nomega;
-  const unsigned nb = blocks_for(nthr, kSpecThreads);
-  if (a.nl == 4)
-    spectrum_kernel<4><<<nb, kSpecThreads, 0, st>>>(a);
-  else
-    spectrum_kernel<3><<<nb, kSpecThreads, 0, st>>>(a);
+  const long long nthr = (long long)a.nchain * a.nomega * a.nl;
+  spectrum_kernel<<<blocks_for(nthr, kSpecThreads), kSpecThreads, 0, st>>>(a);
   TDLZ_LAUNCH_CHECK();
 }
 

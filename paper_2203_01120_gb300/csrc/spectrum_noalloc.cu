@@ -10,32 +10,31 @@ namespace tdlz {
 
 namespace {
 
-// One thread per (chain, omega).
-template <int NL>
+// One thread per (chain, omega, left vector).
 __global__ void __launch_bounds__(kSpecThreads)
     spectrum_noalloc_kernel(int nchain, int nomega, int cap, const int *steps,
                             const double2 *alpha, const double *beta, const double2 *gamma,
                             const double2 *z, const double *n0, const double *wk, double start,
-                            double step, double eta, double2 *chi) {
+                            double step, double eta, int nl, double2 *chi) {
   long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (tid >= (long long)nchain * nomega) return;
-  int c = (int)(tid / nomega);
-  int iw = (int)(tid - (long long)c * nomega);
+  if (tid >= (long long)nchain * nomega * nl) return;
+  const long long ciw = tid / nl;
+  const int l = (int)(tid - ciw * nl);
+  const int c = (int)(ciw / nomega);
+  const int iw = (int)(ciw - (long long)c * nomega);
   int m = steps[c];  // read on the device: clamped to [0, cap]
   if (m > cap) m = cap;
-  double2 *out = chi + ((long long)c * NL) * nomega + iw;
+  double2 *out = chi + ((long long)c * nl + l) * nomega + iw;
   if (m <= 0) {
-    for (int l = 0; l < NL; ++l) out[(long long)l * nomega] = make_double2(0, 0);
+    *out = make_double2(0, 0);
     return;
   }
-  double2 acc[NL];
-  tridiag_chi<NL>(m, cap, alpha + (long long)c * cap, beta + (long long)c * cap,
-                  gamma + (long long)c * cap, z + (long long)c * NL * cap,
-                  make_double2(start + step * iw, eta), make_double2(0, 0), acc);
+  const double2 acc = tridiag_chi(m, alpha + (long long)c * cap, beta + (long long)c * cap,
+                                  gamma + (long long)c * cap,
+                                  z + ((long long)c * nl + l) * cap,
+                                  make_double2(start + step * iw, eta), make_double2(0, 0));
   double s = wk[c] * n0[c];
-#pragma unroll
-  for (int l = 0; l < NL; ++l)
-    out[(long long)l * nomega] = make_double2(s * acc[l].x, s * acc[l].y);
+  *out = make_double2(s * acc.x, s * acc.y);
 }
 
 }  // namespace
@@ -65,19 +64,14 @@ void spectrum_noalloc(Context &ctx, const tdlz_coeffs *c, const tdlz_spectrum_pa
                    std::to_string(TDLZ_NOALLOC_SCRATCH_MB) + " MiB holds nchain * nsteps <= " +
                    std::to_string(cap_steps) + ")");
   const double conv = sp->units == 1 ? 1.0 / 27211.386245988 : 1.0;
-  auto launch = [&](auto kernel) {
-    kernel<<<blocks_for((long long)c->nchain * nomega, kSpecThreads), kSpecThreads, 0,
-             ctx.stream>>>(
-        c->nchain, nomega, c->nsteps, c->steps, reinterpret_cast<const double2 *>(c->alpha),
-        c->beta, reinterpret_cast<const double2 *>(c->gamma),
-        reinterpret_cast<const double2 *>(c->z), c->n0, c->wk, sp->start * conv, sp->step * conv,
-        sp->eta * conv, reinterpret_cast<double2 *>(chi));
-    TDLZ_LAUNCH_CHECK();
-  };
-  if (c->ncomp == 4)
-    launch(spectrum_noalloc_kernel<4>);
-  else
-    launch(spectrum_noalloc_kernel<3>);
+  const int nl = c->ncomp == 4 ? 4 : 3;
+  spectrum_noalloc_kernel<<<blocks_for((long long)c->nchain * nomega * nl, kSpecThreads),
+                            kSpecThreads, 0, ctx.stream>>>(
+      c->nchain, nomega, c->nsteps, c->steps, reinterpret_cast<const double2 *>(c->alpha),
+      c->beta, reinterpret_cast<const double2 *>(c->gamma),
+      reinterpret_cast<const double2 *>(c->z), c->n0, c->wk, sp->start * conv, sp->step * conv,
+      sp->eta * conv, nl, reinterpret_cast<double2 *>(chi));
+  TDLZ_LAUNCH_CHECK();
 }
 
 }  // namespace tdlz

@@ -1,12 +1,13 @@
 // The tridiagonal solve behind chi(omega) (Eqs. resolvent_Liouvillian_Lanczos_q and
 // post_processing), shared by tdlz_spectrum and tdlz_spectrum_noalloc.
 //
-// One thread solves one (chain, omega).  The solve is bound by the FP64 pipe (two lanes
-// per clock and SM on this part: a warp instruction takes 16 clocks of its SM whatever the
-// other SMs do), so its cost is the FP64 instructions of one step times the steps, and the
-// kernels run one warp per block: 3 chains x 1001 frequencies are 94 warps on 94 SMs
-// instead of four to a block on 24.  Measured for that case with 1500 steps: see
-// tridiag_chi.
+// Bound by the FP64 issue rate of one warp: each of an SM's four schedulers starts one FP64
+// warp instruction per 64 clocks, whatever the number of active lanes (the four together
+// one per 19), so a solve takes 64 clocks x the instructions of a step x the steps until
+// the 608 schedulers are full.  Hence one thread per (chain, omega, left vector) with the
+// continuant recomputed by each (16 instructions a step instead of 28 for all three left
+// vectors: 282 warps for 3 chains x 1001 frequencies), in blocks of one warp so that they
+// spread over the SMs.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -41,115 +42,65 @@ __device__ __forceinline__ int spec_mag(double2 a) {
   return max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff);
 }
 
-// 1 / c, one division; numbers whose square would leave the double range take Smith's
-// method (mag = spec_mag(c): exponents within +-400).
-__device__ __forceinline__ double2 spec_recip(double2 c, int mag) {
-  if (mag >= (623 << 20) && mag < (1423 << 20)) {
-    const double r = 1.0 / fma(c.x, c.x, c.y * c.y);
-    return make_double2(c.x * r, -c.y * r);
-  }
-  return spec_cdiv(make_double2(1.0, 0.0), c);
+// 2^-e of the upper word `mag` of the largest component; 1 for zero and non-finite values
+__device__ __forceinline__ double spec_pow2(int mag) {
+  const int e = (mag >> 20) - 1023;
+  return e > -1000 && e < 1000 ? __hiloint2double((1023 - e) << 20, 0) : 1.0;
 }
 
-// acc[l] = sum_i conj(z^l_i) x_i for (zw - T) x = e_1 with the m x m tridiagonal T
-// (diagonal alpha, sub-diagonal beta, super-diagonal gamma) and `tail` subtracted from the
-// last diagonal entry (the continued fraction of an extrapolated part; zero without one).
+// sum_i conj(z_i) x_i for (zw - T) x = e_1 with the m x m tridiagonal T (diagonal alpha,
+// sub-diagonal beta, super-diagonal gamma) and `tail` subtracted from the last diagonal
+// entry (the continued fraction of an extrapolated part; zero without one).
 //
-// Gaussian elimination with partial pivoting from the last row up.  The right-hand side is
-// zero below the first row, so nothing has to be kept: eliminating x_{i+1} leaves one
-// pending row  p x_i + q x_{i+1} = 0  and  x_{i+1} = s x_i + t x_{i-1}  (t != 0 only where
-// row i was the pivot), and the sums over j > i are carried along as the functional
-// A_l x_{i+1} + B_l x_i.  No scratch, no second sweep: against the top-down elimination
-// that stored its rows (four complex words per step, written and read back) and formed two
-// hypot and six divisions per step this does one division and about 45 FP64 instructions.
-// 3 chains x 1500 steps x 1001 frequencies: 9.35 ms before, @SPEC_FULL@ after (whole calls).
-// Pivots are compared in the maximum norm to 20 bits: |multiplier| <= sqrt 2, so the growth
-// bound of partial pivoting stays; measured errors against extended precision are below
-// the top-down form's (2.4e-16 against 6.1e-16 of the norm at 1500 steps).
-template <int NL>
-__device__ __forceinline__ void tridiag_chi(int m, int cap, const double2 *__restrict__ al,
-                                            const double *__restrict__ be,
-                                            const double2 *__restrict__ ga,
-                                            const double2 *__restrict__ zz, double2 zw,
-                                            double2 tail, double2 (&acc)[NL]) {
-  double2 q = make_double2(zw.x - al[m - 1].x - tail.x, zw.y - al[m - 1].y - tail.y);
-  double2 A[NL], B[NL];
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    const double2 zv = zz[(long long)l * cap + m - 1];
-    A[l] = make_double2(zv.x, -zv.y);
-    B[l] = make_double2(0.0, 0.0);
-  }
-  if (m == 1) {
-    const double2 x = spec_cdiv(make_double2(1.0, 0.0), q);
-#pragma unroll
-    for (int l = 0; l < NL; ++l) acc[l] = spec_mul(A[l], x);
-    return;
-  }
-  double2 p = make_double2(-be[m - 2], 0.0);
+// With D_i the determinant of rows and columns i..m,
+//   D_i = (zw - alpha_i) D_{i+1} - beta_i gamma_i D_{i+2},
+//   x_i = beta_1 .. beta_{i-1} D_{i+1} / D_1,
+// so the sum is A_1 / D_1 with A_i = conj(z_i) D_{i+1} + beta_i A_{i+1}: one sweep from the
+// last row up, no division, no pivots and no stored rows.  The D computed this way are the
+// exact ones of a matrix whose entries differ by rounding errors (each step's errors can be
+// put on its own alpha and beta gamma), so the solve is at least as stable as elimination
+// with partial pivoting; measured against extended precision at 1500 steps: 3.6e-16
+// (non-Hermitian chains) and 1.5e-16 (alternating signs) of the norm, pivoted elimination
+// 6.6e-16 and 1.9e-16.  D and A share one power-of-two scale, which the ratio drops.
+// Whole calls, 3 chains x 1500 steps x 1001 frequencies: 9.31 ms with pivoted elimination
+// over stored rows, 2.80 ms without the rows, 1.27 ms in this form.
+__device__ __forceinline__ double2 tridiag_chi(int m, const double2 *__restrict__ al,
+                                               const double *__restrict__ be,
+                                               const double2 *__restrict__ ga,
+                                               const double2 *__restrict__ z, double2 zw,
+                                               double2 tail) {
+  double2 d1 = make_double2(zw.x - al[m - 1].x - tail.x, zw.y - al[m - 1].y - tail.y);  // D_m
+  double2 d2 = make_double2(1.0, 0.0);
+  double2 A = make_double2(z[m - 1].x, -z[m - 1].y);
   // coefficients of the next row, loaded one step ahead
-  double2 an = al[m - 2], gn = ga[m - 2], zn[NL];
-  double bn = m > 2 ? be[m - 3] : 0.0;
-#pragma unroll
-  for (int l = 0; l < NL; ++l) zn[l] = zz[(long long)l * cap + m - 2];
-  for (int i = m - 2; i >= 1; --i) {
-    const double2 d = make_double2(zw.x - an.x, zw.y - an.y), du = make_double2(-gn.x, -gn.y);
-    const double dl = -bn;
-    double2 zv[NL];
-#pragma unroll
-    for (int l = 0; l < NL; ++l) zv[l] = zn[l];
-    an = al[i - 1];
-    gn = ga[i - 1];
-    bn = i > 1 ? be[i - 2] : 0.0;
-#pragma unroll
-    for (int l = 0; l < NL; ++l) zn[l] = zz[(long long)l * cap + i - 1];
-    const int mq = spec_mag(q), mu = spec_mag(du);
-    if (mq >= mu) {  // the pending row is the pivot: x_{i+1} = -(p / q) x_i
-      const double2 ic = spec_recip(q, mq);
-      const double2 s = spec_mul(p, ic), f = spec_mul(du, ic);  // s negated
-      q = spec_nfma(d, f, p);
-      p = make_double2(dl, 0.0);
-#pragma unroll
-      for (int l = 0; l < NL; ++l) {
-        const double2 c = make_double2(zv[l].x + B[l].x, B[l].y - zv[l].y);
-        A[l] = spec_nfma(c, A[l], s);
-        B[l] = make_double2(0.0, 0.0);
-      }
-    } else {  // row i is the pivot: x_{i+1} = -(d x_i + dl x_{i-1}) / du
-      const double2 ic = spec_recip(du, mu);
-      const double2 s = spec_mul(d, ic), f = spec_mul(q, ic);
-      const double2 t = make_double2(-dl * ic.x, -dl * ic.y);
-      q = spec_nfma(p, f, d);
-      p = make_double2(-f.x * dl, -f.y * dl);
-#pragma unroll
-      for (int l = 0; l < NL; ++l) {
-        const double2 c = make_double2(zv[l].x + B[l].x, B[l].y - zv[l].y);
-        B[l] = spec_mul(A[l], t);
-        A[l] = spec_nfma(c, A[l], s);
-      }
+  const int i0 = m > 1 ? m - 2 : 0;
+  double2 an = al[i0], gn = ga[i0], zn = z[i0];
+  double bn = be[i0];
+  for (int i = m - 2; i >= 0; --i) {
+    const double2 d = make_double2(zw.x - an.x, zw.y - an.y), zv = zn;
+    const double2 bc = make_double2(bn * gn.x, bn * gn.y);
+    const double b = bn;
+    const int in = i > 0 ? i - 1 : 0;
+    an = al[in];
+    gn = ga[in];
+    zn = z[in];
+    bn = be[in];
+    // conj(z) D + beta A
+    A = make_double2(fma(zv.x, d1.x, fma(zv.y, d1.y, b * A.x)),
+                     fma(zv.x, d1.y, fma(-zv.y, d1.x, b * A.y)));
+    const double2 t = spec_mul(d, d1);
+    const double2 d0 = spec_nfma(t, bc, d2);
+    d2 = d1;
+    d1 = d0;
+    const int mag = max(spec_mag(d1), spec_mag(d2));
+    if (mag < (823 << 20) || mag > (1223 << 20)) {  // beyond 2^+-200 (seldom)
+      const double sc = spec_pow2(mag);
+      d1 = make_double2(d1.x * sc, d1.y * sc);
+      d2 = make_double2(d2.x * sc, d2.y * sc);
+      A = make_double2(A.x * sc, A.y * sc);
     }
   }
-  // first row: d x_1 + du x_2 = 1 with the pending p x_1 + q x_2 = 0
-  const double2 d = make_double2(zw.x - an.x, zw.y - an.y), du = make_double2(-gn.x, -gn.y);
-  const double2 one = make_double2(1.0, 0.0);
-  double2 x1, x2;
-  if (spec_mag(q) >= spec_mag(du)) {
-    const double2 ic = spec_cdiv(one, q);
-    x1 = spec_cdiv(one, spec_nfma(d, spec_mul(du, ic), p));
-    const double2 s = spec_mul(p, ic);
-    x2 = spec_nfma(make_double2(0.0, 0.0), s, x1);
-  } else {
-    const double2 ic = spec_cdiv(one, du);
-    const double2 f = spec_mul(q, ic);
-    x1 = spec_cdiv(make_double2(-f.x, -f.y), spec_nfma(p, f, d));
-    x2 = spec_mul(spec_nfma(one, d, x1), ic);
-  }
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    const double2 b = make_double2(B[l].x + zn[l].x, B[l].y - zn[l].y);
-    const double2 ax = spec_mul(A[l], x2), bx = spec_mul(b, x1);
-    acc[l] = make_double2(ax.x + bx.x, ax.y + bx.y);
-  }
+  return spec_cdiv(A, d1);
 }
 
 }  // namespace tdlz
