@@ -413,7 +413,7 @@ template <class T, int N1, int N2, int DIR>
 __device__ __forceinline__ int zline_fft(cx<T> (&a)[N2], int n1, const RegTw<T, N2> &tw2,
                                          const RegTw<T, N1 * N2> &twn) {
   constexpr int N = N1 * N2;
-  RegPlan<N2>::template run<T, DIR>(a, tw2);
+  RegPlan<N2>::template run<T, DIR, (DIR > 0)>(a, tw2);
   if constexpr (N1 == 1) {
     return 0;
   } else {
@@ -803,10 +803,15 @@ template <int N> __host__ __device__ constexpr int yx_pstride() {
   return (N * kJ3) % 16 == 8 ? N * kJ3 : N * kJ3 + 8;
 }
 template <int N> constexpr int yx_threads() { return 32 * ((N * kJ3 + 63) / 64); }
-constexpr int kYXMaxThreads = 192;
+// CTAs per SM the register budget is sized for.  36 points, 640 threads per SM at 96
+// registers: inverse 0.505 ms (0.522 at the compiler's own 104-112 registers and three CTAs),
+// forward 0.587 ms (0.664) for one vector of the 36 x 36 x 96 slab with 16 k points.
+template <class T, int N> constexpr int yx_ctas() {
+  return sizeof(T) == 8 ? 1 : N <= 36 ? 4 : 2;
+}
 
 template <class T, int N>
-__global__ void __launch_bounds__(kYXMaxThreads)
+__global__ void __launch_bounds__(yx_threads<N>(), (yx_ctas<T, N>()))
     inv_yx_reg_kernel(const cx<T> *__restrict__ i1, cx<T> *__restrict__ xr,
                       const int *__restrict__ npl, const int *__restrict__ sid,
                       const int *__restrict__ plof, int nk, int nb, int nsm, int npm, int n3,
@@ -861,7 +866,7 @@ __global__ void __launch_bounds__(kYXMaxThreads)
 // Forward: X lines of the box (keeping the sphere's planes) into shared memory, then
 // the Y lines of those planes written to the sphere's sticks.
 template <class T, int N>
-__global__ void __launch_bounds__(kYXMaxThreads)
+__global__ void __launch_bounds__(yx_threads<N>(), (yx_ctas<T, N>()))
     fwd_xy_reg_kernel(const cx<T> *__restrict__ xr, cx<T> *__restrict__ i1,
                       const int *__restrict__ npl, const int *__restrict__ sid,
                       const int *__restrict__ plof, int nk, int nb, int nsm, int npm, int n3,
