@@ -213,4 +213,14 @@ inline unsigned blocks_for(long long n, int t = 256) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
+// Threads per CTA of a pointwise kernel over n points in `rows` block rows: 256, or fewer
+// (down to a warp) while the launch would leave schedulers idle.  An SM's four schedulers
+// each start one FP64 warp instruction per 64 clocks, so a small FP64 launch takes the time
+// of its fullest SM: 4096 points in 16 CTAs of 256 ran on 16 of the 152 SMs.
+inline int spread_threads(long long n, long long rows) {
+  int th = 256;
+  while (th > 32 && (n + th - 1) / th * rows < 4 * 152) th /= 2;
+  return th;
+}
+
 }  // namespace tdlz

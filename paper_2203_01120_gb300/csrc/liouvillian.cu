@@ -63,20 +63,20 @@ inline dim3 row_grid(long long nrows, int npwx) {
 // t = (1,-1,-1,-1); fixed summation order (deterministic).
 // nvec response vectors share the occupied orbitals: each U(r) value is read once
 // and contracted with every vector's x(r); rho is [nvec][4][Nr].
-// Block row y sums the (side, k) pairs [y*ppg, (y+1)*ppg) into partial slice y
+// Block row y sums the band-sides (side, k, n) [y*len, (y+1)*len) into partial slice y
 // ([gridDim.y][nvec][4][Nr]); density_reduce_kernel adds the slices in order.
 template <class T, int NV>
 __global__ void __launch_bounds__(256)
     density_kernel(const cx<T> *__restrict__ ur, const cx<T> *__restrict__ xr,
                    const T *__restrict__ wk, cx<T> *__restrict__ rho, int nk, int nb,
-                   long long nr, int ppg, int vstride) {
+                   long long nr, int len, int vstride) {
   const long long rows1 = 4LL * nk * nb;
-  const int pb = blockIdx.y * ppg, pe = min(2 * nk, pb + ppg);
+  const int i0 = blockIdx.y * len, i1 = min(2 * nk * nb, i0 + len);
   rho += (long long)blockIdx.y * vstride * 4 * nr;
   if constexpr (sizeof(T) == 4) {
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nr;
          r += (long long)gridDim.x * blockDim.x) {
-      // acc[v][a] = sum over the group's (side, k) pairs and bands of w t_a U^+ s_a x, with
+      // acc[v][a] = sum over the group's band-sides of w t_a U^+ s_a x, with
       // t = (1, -1, -1, -1) on the Y side: U is scaled once per band by w t_1 (= +-w), and
       // the charge part (t_0 = 1) takes the same products with the side's sign, so no
       // per-pair partial sums are needed
@@ -85,11 +85,9 @@ __global__ void __launch_bounds__(256)
       for (int v = 0; v < NV; ++v)
 #pragma unroll
         for (int a = 0; a < 4; ++a) acc[v][a] = czero<T>();
-      const int nit = (pe - pb) * nb;
-      // loads of iteration it + 1 issued before the products of iteration it
+      // loads of band-side it + 1 issued before the products of band-side it
       auto load = [&](int it, cx<T> &u0, cx<T> &u1, cx<T> (&x)[NV][2]) {
-        const int pair = pb + it / nb, n = it - (it / nb) * nb;
-        const long long row = ((long long)pair * nb + n) * 2;
+        const long long row = (long long)it * 2;
         u0 = __ldg(ur + row * nr + r);
         u1 = __ldg(ur + (row + 1) * nr + r);
 #pragma unroll
@@ -100,8 +98,8 @@ __global__ void __launch_bounds__(256)
         }
       };
       cx<T> u0, u1, xv[NV][2];
-      if (nit > 0) load(0, u0, u1, xv);
-      for (int it = 0; it < nit; ++it) {
+      if (i0 < i1) load(i0, u0, u1, xv);
+      for (int it = i0; it < i1; ++it) {
         const cx<T> cu0 = u0, cu1 = u1;
         cx<T> cx_[NV][2];
 #pragma unroll
@@ -109,8 +107,8 @@ __global__ void __launch_bounds__(256)
           cx_[v][0] = xv[v][0];
           cx_[v][1] = xv[v][1];
         }
-        if (it + 1 < nit) load(it + 1, u0, u1, xv);
-        const int pair = pb + it / nb;
+        if (it + 1 < i1) load(it + 1, u0, u1, xv);
+        const int pair = it / nb;
         const int side = pair / nk, k = pair - side * nk;
         const T w = wk[k], wt = side == 0 ? w : -w;
         const cx<T> b0 = cscale<T>(cu0, wt), b1 = cscale<T>(cu1, wt);   // magnetic weight
@@ -133,8 +131,11 @@ __global__ void __launch_bounds__(256)
         for (int a = 0; a < 4; ++a) rho[((long long)v * 4 + a) * nr + r] = acc[v][a];
     }
   } else {
-    // FP64 (bound by the FP64 rate): products shared by the charge and magnetic parts,
-    // the k weights applied once per (side, k) pair
+    // FP64 (bound by the FP64 pipe): the four products conj(U_s) x_t accumulate by fused
+    // multiply-adds over the bands of one (side, k) pair, 16 FP64 instructions per band and
+    // vector; the Pauli combinations and the k weight follow once per pair.  Forming the
+    // combinations per band took 32: 2.39 against 1.10 ms for one vector of the 36 x 36 x 96
+    // slab (4 k points, 40 bands).
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nr;
          r += (long long)gridDim.x * blockDim.x) {
       cx<T> acc[NV][4];
@@ -142,35 +143,36 @@ __global__ void __launch_bounds__(256)
       for (int v = 0; v < NV; ++v)
 #pragma unroll
         for (int a = 0; a < 4; ++a) acc[v][a] = czero<T>();
-      for (int pair = pb; pair < pe; ++pair) {
-        const int side = pair / nk, k = pair - side * nk;
-        const T w = wk[k], wt = side == 0 ? w : -w;
-        cx<T> a[NV][4];
+      for (int it = i0; it < i1;) {
+        const int pair = it / nb, side = pair / nk;
+        const T w = wk[pair - side * nk], wt = side == 0 ? w : -w;
+        const int ie = min(i1, (pair + 1) * nb);
+        cx<T> p[NV][4];  // 00, 01, 10, 11
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) a[v][c] = czero<T>();
-        for (int n = 0; n < nb; ++n) {
-          const long long row = ((long long)pair * nb + n) * 2;
+          for (int c = 0; c < 4; ++c) p[v][c] = czero<T>();
+        for (; it < ie; ++it) {
+          const long long row = 2LL * it;
           const cx<T> u0 = __ldg(ur + row * nr + r), u1 = __ldg(ur + (row + 1) * nr + r);
 #pragma unroll
           for (int v = 0; v < NV; ++v) {  // every vector of the pass: no early exit, so
             const long long rv = row + v * rows1;  // all loads of a band issue together
             const cx<T> x0 = xr[rv * nr + r], x1 = xr[(rv + 1) * nr + r];
-            const cx<T> p00 = cmulc<T>(u0, x0), p01 = cmulc<T>(u0, x1);
-            const cx<T> p10 = cmulc<T>(u1, x0), p11 = cmulc<T>(u1, x1);
-            a[v][0] = cadd<T>(a[v][0], cadd<T>(p00, p11));
-            a[v][1] = cadd<T>(a[v][1], cadd<T>(p01, p10));
-            const cx<T> d = csub<T>(p10, p01);  // m_y: i (p10 - p01)
-            a[v][2] = cadd<T>(a[v][2], mk<T>(-d.y, d.x));
-            a[v][3] = cadd<T>(a[v][3], csub<T>(p00, p11));
+            cfmac<T>(p[v][0], u0, x0);
+            cfmac<T>(p[v][1], u0, x1);
+            cfmac<T>(p[v][2], u1, x0);
+            cfmac<T>(p[v][3], u1, x1);
           }
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          acc[v][0] = cadd<T>(acc[v][0], cscale<T>(a[v][0], w));
-#pragma unroll
-          for (int c = 1; c < 4; ++c) acc[v][c] = cadd<T>(acc[v][c], cscale<T>(a[v][c], wt));
+          const cx<T> n = cadd<T>(p[v][0], p[v][3]), m1 = cadd<T>(p[v][1], p[v][2]);
+          const cx<T> d = csub<T>(p[v][2], p[v][1]), m3 = csub<T>(p[v][0], p[v][3]);
+          acc[v][0] = mk<T>(fma(w, n.x, acc[v][0].x), fma(w, n.y, acc[v][0].y));
+          acc[v][1] = mk<T>(fma(wt, m1.x, acc[v][1].x), fma(wt, m1.y, acc[v][1].y));
+          acc[v][2] = mk<T>(fma(-wt, d.y, acc[v][2].x), fma(wt, d.x, acc[v][2].y));
+          acc[v][3] = mk<T>(fma(wt, m3.x, acc[v][3].x), fma(wt, m3.y, acc[v][3].y));
         }
       }
 #pragma unroll
@@ -198,20 +200,21 @@ constexpr int kDensityGroups = 8;
 template <class T>
 void density_passes(cudaStream_t st, const cx<T> *ur, const cx<T> *xr, const T *wk, cx<T> *rho,
                     cx<T> *part, int nk, int nb, long long nr, int nvec, int per, dim3 grid,
-                    int ppg, int ng, long long rows1);
+                    int th, int len, int ng, long long rows1);
 
 template <class T>
 void launch_density(Context &ctx, const cx<T> *ur, const cx<T> *xr, const T *wk, cx<T> *rho,
                     cx<T> *part, int nk, int nb, long long nr, int nvec) {
   cudaStream_t st = ctx.stream;
-  // (side, k) pairs split over kDensityGroups block rows for parallelism; up to 3
+  // band-sides split over kDensityGroups block rows for parallelism; up to 3
   // vectors per pass (register budget), each sharing the U(r) reads
   const long long rows1 = 4LL * nk * nb;
-  const int npair = 2 * nk;
-  const int ngroup = std::min(kDensityGroups, npair);
-  const int ppg = (npair + ngroup - 1) / ngroup;
-  const int ng = (npair + ppg - 1) / ppg;
-  const dim3 grid(blocks_for(nr), ng);
+  const int nbs = 2 * nk * nb;
+  const int ngroup = std::min(kDensityGroups, nbs);
+  const int len = (nbs + ngroup - 1) / ngroup;
+  const int ng = (nbs + len - 1) / len;
+  const int th = spread_threads(nr, ng);
+  const dim3 grid(blocks_for(nr, th), ng);
   // vectors per pass (2 or 3, autotuned; 3 is the default): each pass reads U(r) once,
   // more vectors per pass raise the register count.  Each vector's sums run in the
   // same order whatever the grouping, so the choice changes no result.
@@ -220,23 +223,23 @@ void launch_density(Context &ctx, const cx<T> *ur, const cx<T> *xr, const T *wk,
            sizeof(T) == 4 ? "f32" : "f64", nr, rows1, nvec);
   ctx.tuner.pick(st, key, nvec > 1 ? std::vector<int>{2, 3} : std::vector<int>{3}, 3,
                  [&](int per) { density_passes<T>(st, ur, xr, wk, rho, part, nk, nb, nr, nvec,
-                                                  per, grid, ppg, ng, rows1); });
+                                                  per, grid, th, len, ng, rows1); });
 }
 
 template <class T>
 void density_passes(cudaStream_t st, const cx<T> *ur, const cx<T> *xr, const T *wk, cx<T> *rho,
                     cx<T> *part, int nk, int nb, long long nr, int nvec, int per, dim3 grid,
-                    int ppg, int ng, long long rows1) {
+                    int th, int len, int ng, long long rows1) {
   for (int v0 = 0; v0 < nvec; v0 += per) {
     const int nv = std::min(per, nvec - v0);
     const cx<T> *xv = xr + (long long)v0 * rows1 * nr;
     cx<T> *pv = part + (long long)v0 * 4 * nr;
     if (nv == 1)
-      density_kernel<T, 1><<<grid, kThreads, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, ppg, nvec);
+      density_kernel<T, 1><<<grid, th, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, len, nvec);
     else if (nv == 2)
-      density_kernel<T, 2><<<grid, kThreads, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, ppg, nvec);
+      density_kernel<T, 2><<<grid, th, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, len, nvec);
     else
-      density_kernel<T, 3><<<grid, kThreads, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, ppg, nvec);
+      density_kernel<T, 3><<<grid, th, 0, st>>>(ur, xv, wk, pv, nk, nb, nr, len, nvec);
     TDLZ_LAUNCH_CHECK();
   }
   long long n = (long long)nvec * 4 * nr;
@@ -250,6 +253,9 @@ template <class T>
 __global__ void potential_kernel(const cx<T> *__restrict__ rho, const cx<T> *__restrict__ vh,
                                  const T *__restrict__ f, cx<T> *__restrict__ v, long long nr,
                                  int use_h, int use_xc) {
+  rho += blockIdx.y * 4LL * nr;  // this block row's vector
+  vh += blockIdx.y * nr;
+  v += blockIdx.y * 4LL * nr;
   for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nr;
        r += (long long)gridDim.x * blockDim.x) {
     cx<T> out[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};
@@ -1264,12 +1270,10 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
         if (use_h) hartree(m);
         ProfScope ps(pf, st, ST_POTENTIAL, m * (9 * nr * c + 10 * nr * re),
                      16.0 * 4 * nr * m);
-        for (int v = 0; v < m; ++v) {
-          potential_kernel<T><<<blocks_for(nr), kThreads, 0, st>>>(
-              rho + (long long)v * 4 * nr, hg + (long long)v * nr, d.fxc.template as<T>(),
-              vp + (long long)v * 4 * nr, nr, use_h ? 1 : 0, use_xc ? 1 : 0);
-          TDLZ_LAUNCH_CHECK();
-        }
+        const int th = spread_threads(nr, m);
+        potential_kernel<T><<<dim3(blocks_for(nr, th), m), th, 0, st>>>(
+            rho, hg, d.fxc.template as<T>(), vp, nr, use_h ? 1 : 0, use_xc ? 1 : 0);
+        TDLZ_LAUNCH_CHECK();
       } else {
         TDLZ_CUDA_TRY(cudaMemsetAsync(vp, 0, w.vpot.bytes, st));
       }
