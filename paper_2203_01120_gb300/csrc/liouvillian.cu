@@ -283,67 +283,121 @@ __global__ void potential_kernel(const cx<T> *__restrict__ rho, const cx<T> *__r
 
 // ------------------------------------------------------------------ GEMMs
 // Split-K reduction GEMM: part[z][b][m][n] = sum_{k in split z} conj(A[bA][m][k]) B[b][n][k].
-// 16 x 16 threads, each holding an R x R register tile (rows ty + 16 i, columns
-// tx + 16 j), so one CTA covers a (16 R) x (16 R) output tile: per shared-memory
-// load a thread does R complex multiply-adds.
+// TY x TX threads, each holding an RM x RN register tile (rows ty + TY i, columns
+// tx + TX j), so one CTA covers a (TY RM) x (TX RN) output tile: per shared-memory
+// load a thread does about R complex multiply-adds.  Shape and split: tn_shape.
 constexpr int KC = 16;
-template <class T, int R>
+template <class T, int RM, int RN>
 __global__ void __launch_bounds__(256)
     gemm_tn_kernel(const cx<T> *__restrict__ A, long long lda, long long sA, int amod,
                    const cx<T> *__restrict__ B, long long ldb, long long sB,
-                   cx<T> *__restrict__ part, int M, int N, long long K, int batch, int nsplit) {
-  constexpr int TT = 16 * R;
-  __shared__ cx<T> As[TT][KC + 1];
-  __shared__ cx<T> Bs[TT][KC + 1];
+                   cx<T> *__restrict__ part, int M, int N, long long K, int batch, int nsplit,
+                   int TY, int TX) {
+  extern __shared__ unsigned char tn_smem[];
+  const int TM = TY * RM, TN = TX * RN;
+  cx<T>(*As)[KC + 1] = reinterpret_cast<cx<T>(*)[KC + 1]>(tn_smem);
+  cx<T>(*Bs)[KC + 1] = As + TM;
   int z = blockIdx.z;
   int b = z % batch;
   int sp = z / batch;
-  int m0 = blockIdx.y * TT, n0 = blockIdx.x * TT;
+  int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
   long long kchunk = (K + nsplit - 1) / nsplit;
   long long kb = sp * kchunk, ke = kb + kchunk < K ? kb + kchunk : K;
   const cx<T> *Ab = A + (long long)(b % amod) * sA;
   const cx<T> *Bb = B + (long long)b * sB;
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  cx<T> acc[R][R];
+  const int ty = threadIdx.x / TX, tx = threadIdx.x - ty * TX;
+  const bool on = ty < TY;  // the last warp may be partly idle
+  cx<T> acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < R; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < R; ++j) acc[i][j] = czero<T>();
+    for (int j = 0; j < RN; ++j) acc[i][j] = czero<T>();
   for (long long k0 = kb; k0 < ke; k0 += KC) {
-    for (int e = threadIdx.x; e < TT * KC; e += blockDim.x) {
+    for (int e = threadIdx.x; e < (TM + TN) * KC; e += blockDim.x) {
       int rr = e / KC, kk = e % KC;
       long long kg = k0 + kk;
-      cx<T> av = czero<T>(), bv = czero<T>();
+      cx<T> v = czero<T>();
       if (kg < ke) {
-        if (m0 + rr < M) av = Ab[(long long)(m0 + rr) * lda + kg];
-        if (n0 + rr < N) bv = Bb[(long long)(n0 + rr) * ldb + kg];
+        if (rr < TM) {
+          if (m0 + rr < M) v = Ab[(long long)(m0 + rr) * lda + kg];
+        } else if (n0 + rr - TM < N) {
+          v = Bb[(long long)(n0 + rr - TM) * ldb + kg];
+        }
       }
-      As[rr][kk] = av;
-      Bs[rr][kk] = bv;
+      As[rr][kk] = v;
     }
     __syncthreads();
+    if (on) {
 #pragma unroll 4
-    for (int kk = 0; kk < KC; ++kk) {
-      cx<T> av[R], bv[R];
+      for (int kk = 0; kk < KC; ++kk) {
+        cx<T> av[RM], bv[RN];
 #pragma unroll
-      for (int i = 0; i < R; ++i) av[i] = As[ty + 16 * i][kk];
+        for (int i = 0; i < RM; ++i) av[i] = As[ty + TY * i][kk];
 #pragma unroll
-      for (int j = 0; j < R; ++j) bv[j] = Bs[tx + 16 * j][kk];
+        for (int j = 0; j < RN; ++j) bv[j] = Bs[tx + TX * j][kk];
 #pragma unroll
-      for (int i = 0; i < R; ++i)
+        for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < R; ++j) cfmac<T>(acc[i][j], av[i], bv[j]);
+          for (int j = 0; j < RN; ++j) cfmac<T>(acc[i][j], av[i], bv[j]);
+      }
     }
     __syncthreads();
   }
+  if (!on) return;
 #pragma unroll
-  for (int i = 0; i < R; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < R; ++j) {
-      int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
+    for (int j = 0; j < RN; ++j) {
+      int m = m0 + ty + TY * i, n = n0 + tx + TX * j;
       if (m < M && n < N)
         part[(((long long)sp * batch + b) * M + m) * N + n] = acc[i][j];
     }
+}
+
+// Issue clocks of `warps` equal warps of `instr` FP64 instructions each: a scheduler starts
+// one per 64 clocks, an SM with four busy schedulers one per 19.
+double fp64_clocks(double warps, double instr) {
+  return instr * std::max(64.0, 19.0 * std::ceil(warps / 152.0));
+}
+
+// Register tile, threads and K split of gemm_tn: the candidate with the fewest FP64 issue
+// clocks (whole warps of padded tiles, plus a fixed cost per K tile and the split's
+// reduction).  Small outputs then get small tiles and many short splits (8 x 8 over 610:
+// 90 us of P_c in the 16^3 cell with one 16 x 16 tile and 2 splits, 31 us now), and large ones a
+// tile that divides them (40 x 40 and 64 x 80 in 48 x 48 and 80 x 80 tiles did 1.44 and 1.25
+// times the work: V_NL 4.63 -> 3.17 ms, P_c 2.57 -> 2.17 ms for one vector of the
+// 36 x 36 x 96 slab at 4 k points, updates included).  The FP32 fallback takes the same shapes.
+struct TnShape {
+  int rm = 1, rn = 1, ty = 1, tx = 1, ntm = 1, ntn = 1, nsplit = 1;
+};
+constexpr int kTnTiles[][2] = {{1, 1}, {2, 2}, {3, 3}, {4, 4}, {5, 5}, {4, 5}, {5, 4}};
+TnShape tn_shape(int M, int N, long long K, int batch) {
+  TnShape best;
+  double tbest = -1.0;
+  for (const auto &r : kTnTiles) {
+    TnShape c;
+    c.rm = r[0];
+    c.rn = r[1];
+    const int um = (M + c.rm - 1) / c.rm, un = (N + c.rn - 1) / c.rn;
+    c.ntm = (um + 15) / 16;
+    c.ntn = (un + 15) / 16;
+    c.ty = (um + c.ntm - 1) / c.ntm;
+    c.tx = (un + c.ntn - 1) / c.ntn;
+    const double warps = (double)batch * c.ntm * c.ntn * ((c.ty * c.tx + 31) / 32);
+    for (c.nsplit = 1; c.nsplit <= 32 && (c.nsplit == 1 || K / c.nsplit >= KC); c.nsplit *= 2) {
+      const double kch = (double)((K + c.nsplit - 1) / c.nsplit);
+      // staging and shared-memory loads per product fall with the register tile
+      const double t = fp64_clocks(warps * c.nsplit, 4.0 * c.rm * c.rn * kch) *
+                           (1.0 + 0.05 / c.rm + 0.05 / c.rn) +
+                       600.0 * kch / KC +
+                       fp64_clocks((double)batch * M * N / 32.0, 2.0 * c.nsplit);
+      if (tbest < 0.0 || t < tbest) {
+        tbest = t;
+        best = c;
+      }
+    }
+  }
+  return best;
 }
 
 // C[b*sC + m*ldcm + n*ldcn] = sum_z part[z][b][m][n] (fixed order)
@@ -364,35 +418,36 @@ __global__ void split_reduce_kernel(const cx<T> *__restrict__ part, cx<T> *__res
 }
 
 // Out[b][row][col] = sgn_b (In[b][row][col] + alpha sum_k A(b,row,k) B[b % bmod][k][col])
-constexpr int NN_ROWS = 16, NN_COLS = 128, NN_KMAX = 256;
+constexpr int NN_KMAX = 256;
 // grid: x = row chunk (fastest, so the CTAs that share a B column tile run together
 // and re-read it from L2), y = column chunk, z = batch; A chunk in dynamic smem.
-// Each thread owns NC columns (tid + j NN_COLS, coalesced for every j), so every
-// shared-memory load of A feeds NC complex multiply-adds.
-template <class T, int NC>
-__global__ void __launch_bounds__(NN_COLS)
+// Each thread owns NC columns (tid + j blockDim, coalesced for every j) of NR rows, so
+// every shared-memory load of A feeds NC complex multiply-adds.
+template <class T, int NC, int NR>
+__global__ void __launch_bounds__(128)
     gemm_nn_kernel(const cx<T> *__restrict__ A, long long sA, long long sar, long long sak,
                    const cx<T> *__restrict__ B, long long ldb, long long sB, int bmod,
                    const cx<T> *In, cx<T> *Out, long long ldo, long long sO, int rows,
                    long long ncol, int K, T alpha, int neg_from, int neg_mod) {
   extern __shared__ unsigned char nn_smem[];
-  cx<T> *As = reinterpret_cast<cx<T> *>(nn_smem);  // [NN_ROWS][K]
+  cx<T> *As = reinterpret_cast<cx<T> *>(nn_smem);  // [NR][K]
   int b = blockIdx.z;
-  int r0 = blockIdx.x * NN_ROWS;
+  int r0 = blockIdx.x * NR;
+  const int bd = blockDim.x;
   const cx<T> *Ab = A + (long long)b * sA;
-  for (int e = threadIdx.x; e < NN_ROWS * K; e += blockDim.x) {
+  for (int e = threadIdx.x; e < NR * K; e += bd) {
     int rr = e / K, kk = e % K;
     As[e] = (r0 + rr < rows) ? Ab[(long long)(r0 + rr) * sar + (long long)kk * sak] : czero<T>();
   }
   __syncthreads();
-  const long long col0 = (long long)blockIdx.y * NN_COLS * NC + threadIdx.x;
+  const long long col0 = (long long)blockIdx.y * bd * NC + threadIdx.x;
   if (col0 >= ncol) return;
   const cx<T> *Bb = B + (long long)(b % bmod) * sB;
-  cx<T> acc[NC][NN_ROWS];
+  cx<T> acc[NC][NR];
 #pragma unroll
   for (int j = 0; j < NC; ++j)
 #pragma unroll
-    for (int r = 0; r < NN_ROWS; ++r) acc[j][r] = czero<T>();
+    for (int r = 0; r < NR; ++r) acc[j][r] = czero<T>();
   // B columns prefetched 4 entries at a time (independent loads in flight)
   constexpr int U = 4;
   for (int kk = 0; kk < K; kk += U) {
@@ -401,7 +456,7 @@ __global__ void __launch_bounds__(NN_COLS)
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int j = 0; j < NC; ++j) {
-        const long long c = col0 + j * NN_COLS;
+        const long long c = col0 + j * bd;
         bv[u][j] = (kk + u < K && c < ncol) ? __ldg(Bb + (long long)(kk + u) * ldb + c)
                                             : czero<T>();
       }
@@ -409,26 +464,51 @@ __global__ void __launch_bounds__(NN_COLS)
     for (int u = 0; u < U; ++u) {
       if (kk + u >= K) break;
 #pragma unroll
-      for (int r = 0; r < NN_ROWS; ++r) {
+      for (int r = 0; r < NR; ++r) {
         const cx<T> av = As[r * K + kk + u];
 #pragma unroll
         for (int j = 0; j < NC; ++j) cfma<T>(acc[j][r], av, bv[u][j]);
       }
     }
   }
-  T sg = (b % neg_mod) >= neg_from ? T(-1) : T(1);
+  const bool neg = (b % neg_mod) >= neg_from;
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
-    const long long col = col0 + j * NN_COLS;
+    const long long col = col0 + j * bd;
     if (col >= ncol) break;
 #pragma unroll
-    for (int r = 0; r < NN_ROWS; ++r) {
+    for (int r = 0; r < NR; ++r) {
       if (r0 + r >= rows) break;
       long long o = (long long)b * sO + (long long)(r0 + r) * ldo + col;
       cx<T> iv = In[o];
-      Out[o] = mk<T>(sg * (iv.x + alpha * acc[j][r].x), sg * (iv.y + alpha * acc[j][r].y));
+      const cx<T> h = mk<T>(fma(alpha, acc[j][r].x, iv.x), fma(alpha, acc[j][r].y, iv.y));
+      Out[o] = neg ? mk<T>(-h.x, -h.y) : h;
     }
   }
+}
+
+// Rows per thread of the FP64 update, by the same measure as tn_shape: a chunk that divides
+// the rows (40 rows in chunks of 16 did 1.2 times the work, 70 rows 1.14 times), small
+// chunks where there are few columns.
+struct NnShape {
+  int nr = 16, threads = 128;
+};
+constexpr int kNnRows[] = {16, 14, 12, 10, 8, 4};
+NnShape nn_shape(int rows, long long ncol, int K, int batch) {
+  NnShape best;
+  double tbest = -1.0;
+  for (int nr : kNnRows) {
+    const double warps =
+        (double)batch * ((rows + nr - 1) / nr) * (double)((ncol + 31) / 32);
+    // 2 nr instructions of the epilogue; 3% per row chunk for re-reading B
+    const double t = fp64_clocks(warps, nr * (4.0 * K + 2.0)) * (1.0 + 0.3 / nr);
+    if (tbest < 0.0 || t < tbest) {
+      tbest = t;
+      best.nr = nr;
+      best.threads = warps >= 8 * 608 ? 128 : 32;
+    }
+  }
+  return best;
 }
 
 // dmix[b][(n,s)][i] = sum_{j,t} D[2i+s][2j+t] proj[b][j][(n,t)], over the nonzero
@@ -462,28 +542,31 @@ template <class T>
 void gemm_tn(Context &ctx, DevBuf &partbuf, const cx<T> *A, long long lda, long long sA, int amod,
              const cx<T> *B, long long ldb, long long sB, cx<T> *C, long long sC, long long ldcm,
              long long ldcn, int M, int N, long long K, int batch) {
-  // register tile R (CTA tile 16 R) from the larger output dimension, at most 5 (80)
-  const int R = std::max(1, std::min(5, (std::max(M, N) + 15) / 16));
-  const int TT = 16 * R;
-  const int tiles = ((M + TT - 1) / TT) * ((N + TT - 1) / TT);
-  // enough CTAs to fill the GPU: split K so that batch * tiles * nsplit >= ~4 waves
-  long long want = (4LL * 152 + (long long)batch * tiles - 1) / ((long long)batch * tiles);
-  long long ns = std::min(want, (K + 255) / 256);
-  int nsplit = (int)std::max(1LL, std::min(ns, 32LL));
+  const TnShape c = tn_shape(M, N, K, batch);
+  const int nsplit = c.nsplit;
   size_t need = (size_t)nsplit * batch * M * N * sizeof(cx<T>);
   TDLZ_REQUIRE(need <= partbuf.bytes, TDLZ_ERR_STATE, "split-K scratch too small");
-  dim3 grid((N + TT - 1) / TT, (M + TT - 1) / TT, (unsigned)(batch * nsplit));
+  const dim3 grid(c.ntn, c.ntm, (unsigned)(batch * nsplit));
+  const int threads = (c.ty * c.tx + 31) / 32 * 32;
+  const size_t sm = (size_t)(c.ty * c.rm + c.tx * c.rn) * (KC + 1) * sizeof(cx<T>);
   cx<T> *pp = partbuf.template as<cx<T>>();
-  switch (R) {
-    case 1: gemm_tn_kernel<T, 1><<<grid, 256, 0, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch, nsplit); break;
-    case 2: gemm_tn_kernel<T, 2><<<grid, 256, 0, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch, nsplit); break;
-    case 3: gemm_tn_kernel<T, 3><<<grid, 256, 0, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch, nsplit); break;
-    case 4: gemm_tn_kernel<T, 4><<<grid, 256, 0, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch, nsplit); break;
-    default: gemm_tn_kernel<T, 5><<<grid, 256, 0, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch, nsplit); break;
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, threads, sm, ctx.stream>>>(A, lda, sA, amod, B, ldb, sB, pp, M, N, K, batch,
+                                              nsplit, c.ty, c.tx);
+  };
+  switch (c.rm * 8 + c.rn) {  // at most 160 rows of 17 elements: 43.5 KB in FP64
+    case 9: launch(gemm_tn_kernel<T, 1, 1>); break;
+    case 18: launch(gemm_tn_kernel<T, 2, 2>); break;
+    case 27: launch(gemm_tn_kernel<T, 3, 3>); break;
+    case 36: launch(gemm_tn_kernel<T, 4, 4>); break;
+    case 37: launch(gemm_tn_kernel<T, 4, 5>); break;
+    case 44: launch(gemm_tn_kernel<T, 5, 4>); break;
+    default: launch(gemm_tn_kernel<T, 5, 5>); break;
   }
   TDLZ_LAUNCH_CHECK();
   long long tot = (long long)batch * M * N;
-  split_reduce_kernel<T><<<blocks_for(tot), kThreads, 0, ctx.stream>>>(
+  const int th = spread_threads(tot, 1);
+  split_reduce_kernel<T><<<blocks_for(tot, th), th, 0, ctx.stream>>>(
       partbuf.template as<cx<T>>(), C, M, N, batch, nsplit, sC, ldcm, ldcn);
   TDLZ_LAUNCH_CHECK();
 }
@@ -494,17 +577,29 @@ void gemm_nn(Context &ctx, const cx<T> *A, long long sA, long long sar, long lon
              long long ldo, long long sO, int rows, long long ncol, int K, T alpha, int batch,
              int neg_from, int neg_mod = 1 << 30) {
   TDLZ_REQUIRE(K <= NN_KMAX, TDLZ_ERR_ARG, "contraction length above 256 (nocc or nproj)");
-  // two columns per thread in FP32, one in FP64 (register budget)
-  constexpr int NC = sizeof(T) == 4 ? 2 : 1;
-  dim3 grid((rows + NN_ROWS - 1) / NN_ROWS, (unsigned)((ncol + NN_COLS * NC - 1) / (NN_COLS * NC)),
-            batch);
-  size_t sm = (size_t)NN_ROWS * K * sizeof(cx<T>);
-  TDLZ_CUDA_TRY(cudaFuncSetAttribute(gemm_nn_kernel<T, NC>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  gemm_nn_kernel<T, NC><<<grid, NN_COLS, sm, ctx.stream>>>(A, sA, sar, sak, B, ldb, sB, bmod, In,
-                                                         Out, ldo, sO, rows, ncol, K, alpha,
-                                                         neg_from, neg_mod);
-  TDLZ_LAUNCH_CHECK();
+  auto launch = [&](auto kernel, int nc, int nr, int threads) {
+    const dim3 grid((rows + nr - 1) / nr, (unsigned)((ncol + threads * nc - 1) / (threads * nc)),
+                    batch);
+    const size_t sm = (size_t)nr * K * sizeof(cx<T>);
+    TDLZ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sm));
+    kernel<<<grid, threads, sm, ctx.stream>>>(A, sA, sar, sak, B, ldb, sB, bmod, In, Out, ldo,
+                                              sO, rows, ncol, K, alpha, neg_from, neg_mod);
+    TDLZ_LAUNCH_CHECK();
+  };
+  if constexpr (sizeof(T) == 4) {  // two columns per thread
+    launch(gemm_nn_kernel<T, 2, 16>, 2, 16, 128);
+  } else {
+    const NnShape c = nn_shape(rows, ncol, K, batch);
+    switch (c.nr) {
+      case 4: launch(gemm_nn_kernel<T, 1, 4>, 1, 4, c.threads); break;
+      case 8: launch(gemm_nn_kernel<T, 1, 8>, 1, 8, c.threads); break;
+      case 10: launch(gemm_nn_kernel<T, 1, 10>, 1, 10, c.threads); break;
+      case 12: launch(gemm_nn_kernel<T, 1, 12>, 1, 12, c.threads); break;
+      case 14: launch(gemm_nn_kernel<T, 1, 14>, 1, 14, c.threads); break;
+      default: launch(gemm_nn_kernel<T, 1, 16>, 1, 16, c.threads); break;
+    }
+  }
 }
 
 // ------------------------------------------------- precision conversion
