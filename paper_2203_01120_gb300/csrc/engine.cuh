@@ -136,14 +136,17 @@ struct QSlot {
   DevBuf pl_j1;   // [nk][nplane_max] grid index j1 of each plane
   DevBuf pl_of;   // [nk][n1] plane index of j1 or -1
   DevBuf st_id;   // [nk][nplane_max][n2] stick index of (plane, j2) or -1
+  // slab stages (slab.cu): planes of every k are one run of Miller indices m1 (grid indices
+  // 0 .. x-1 and the last y - x), stick -> plane (n2 + 1) + j2
+  bool slab_planes = false;
+  DevBuf slab_pl;   // [nk] int2 (planes from j1 = 0 up, planes in all)
+  DevBuf slab_pos;  // [nk][nstick_max]
+  bool slab32 = false;  // the FP32 Liouvillian's steps 1-6 run the slab stages
   int dnl_w = 0;   // nonzeros per row of D in the ELL form (padded)
   DevBuf dnl_col;  // [2nproj][dnl_w] column of each entry of dnl_val, -1 past the row's end
   // the Liouvillian of each precision runs the fused plane stages (planes.cu); otherwise
   // the staged pipeline with real-space grids in HBM (pipeline.cu)
   bool planes32 = false, planes64 = false;
-  // the staged pipeline's Y and X line passes of each precision run fused (no plane
-  // buffer in HBM; TDLZ_YX_FUSED=0 keeps the separate passes)
-  bool yx32 = false, yx64 = false;
   // loaded for mixed precision only (TDLZ_MIXED_ONLY=1): the FP32 data is built at load
   // and the FP64 real-space orbitals are released; FP64 applications are refused
   bool mixed_only = false;

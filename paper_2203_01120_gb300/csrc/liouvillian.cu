@@ -25,6 +25,7 @@
 #include "engine.cuh"
 #include "pipeline.cuh"
 #include "planes.cuh"
+#include "slab.cuh"
 #include "tc_gemm.cuh"
 
 namespace tdlz {
@@ -710,9 +711,9 @@ __global__ void sigma_u_kernel(const cx<T> *__restrict__ ck, const int *__restri
 // Bytes of the staged pipeline's buffers for one stacked vector: the real-space grids,
 // the plane buffer and the stick buffer of every row, complex elements of c bytes.
 double staged_vector_bytes(const QSlot &s, size_t c) {
-  const bool fused = c == sizeof(float2) ? s.yx32 : s.yx64;
-  const double per_row = (double)s.nr +
-                         (fused ? 0.0 : (double)s.nplane_max * s.fft[1] * s.fft[2]) +
+  if (c == sizeof(float2) && s.slab32)
+    return (double)s.rows() * s.fft[2] * (planes_nnp(s) + s.nstick_max) * (double)c;
+  const double per_row = (double)s.nr + (double)s.nplane_max * s.fft[1] * s.fft[2] +
                          (double)s.nstick_max * s.fft[2];
   return (double)s.rows() * per_row * (double)c;
 }
@@ -772,15 +773,16 @@ void alloc_workspace(QSlot &s, int nvec) {
     w.i1.reset();
     const size_t ns = (size_t)staged_cap(s, c, nvec);
     w.ns_cap = (int)ns;
-    const bool fused = sizeof(T) == 4 ? s.yx32 : s.yx64;
-    w.xr.alloc(ns * s.rows() * s.nr * c);
-    if (fused)
-      w.i2.reset();  // the fused Y + X passes keep the planes on chip
+    const bool slab = sizeof(T) == 4 && s.slab32;
+    w.xr.alloc(ns * s.rows() * (slab ? s.fft[2] * (size_t)planes_nnp(s) : (size_t)s.nr) * c);
+    if (slab)
+      w.i2.reset();  // the slab stages keep the planes on chip
     else
       w.i2.alloc(ns * s.rows() * s.nplane_max * s.fft[1] * s.fft[2] * c);
     w.i1.alloc(ns * s.rows() * s.nstick_max * s.fft[2] * c);
-    w.rhopart.alloc((size_t)kDensityGroups * ns * 4 * (size_t)s.nr * c);
-    w.vpot.alloc(ns * 4 * (size_t)s.nr * c);
+    w.rhopart.alloc((size_t)(slab ? slab_density_chunks(s) : kDensityGroups) * ns * 4 *
+                    (size_t)s.nr * c);
+    w.vpot.alloc(ns * (slab ? 6 : 4) * (size_t)s.nr * c);
     w.rho.alloc(ns * 4 * (size_t)s.nr * c);
     w.hgrid.alloc(ns * (size_t)s.nr * c);
   }
@@ -1058,10 +1060,10 @@ void load_slot(Context &ctx, QSlot &s, const tdlz_ground_state *gs) {
     s.dev_total = total_b;
     const char *sub_env = std::getenv("TDLZ_STAGED_SUB");
     s.staged_sub_env = sub_env ? std::max(0, std::atoi(sub_env)) : 0;
-    const char *yx_env = std::getenv("TDLZ_YX_FUSED");
-    const bool yx_on = !(yx_env && yx_env[0] == '0');
-    s.yx32 = yx_on && yx_fused_supported<float>(s);
-    s.yx64 = yx_on && yx_fused_supported<double>(s);
+    // FP32: the slab stages (grids in plane order, density and products fused with the line
+    // transforms) take the place of the staged pipeline's line passes wherever the grid
+    // allows them; they decide the bytes of a vector below
+    s.slab32 = slab_supported(s);
     const char *pl_env = std::getenv("TDLZ_PLANES");
     auto want_planes = [&](size_t c) {
       bool want = staged_vector_bytes(s, c) > 0.3 * (double)total_b;
@@ -1070,6 +1072,7 @@ void load_slot(Context &ctx, QSlot &s, const tdlz_ground_state *gs) {
       return want;
     };
     s.planes32 = want_planes(sizeof(float2)) && planes_supported<float>(s);
+    if (s.planes32) s.slab32 = false;
     s.planes64 = want_planes(sizeof(double2)) && planes_supported<double>(s);
   }
   // TDLZ_TC=0 keeps the V_NL / P_c reductions and updates on the CUDA-core GEMMs (A/B timing)
@@ -1206,7 +1209,7 @@ void ensure_precision(Context &ctx, QSlot &s) {
     if (!f.ready) {
       SlotData<double> &d = s.d64;
       convert_buf<float>(ctx, d.ukq, f.ukq);
-      if (s.planes32) {
+      if (s.planes32 || s.slab32) {
         if (d.us.p)
           convert_buf<float>(ctx, d.us, f.us);  // same slab layout
         else
@@ -1244,6 +1247,61 @@ void ensure_precision(Context &ctx, QSlot &s) {
 }
 
 // ==================================================================== apply
+// Steps 1-6 of nv stacked vectors on the slab stages; x and h are the first vector's.
+template <class H>
+void slab_stages(Context &ctx, QSlot &s, SlotData<float> &d, Workspace<float> &w,
+                 const float2 *x, float2 *h, int nv, bool use_h, bool use_xc, H &&hartree) {
+  Profiler &pf = ctx.prof;
+  cudaStream_t st = ctx.stream;
+  const int n2 = s.fft[1], n3 = s.fft[2];
+  float2 *i1 = w.i1.as<float2>(), *xs = w.xr.as<float2>(), *rho = w.rho.as<float2>();
+  float2 *hg = w.hgrid.as<float2>();
+  float4 *vp = w.vpot.as<float4>();
+  const float2 *us = d.us.as<float2>();
+  double st_rows = 0, yx_lines = 0;
+  for (int k = 0; k < s.nk; ++k) {
+    st_rows += 4.0 * s.nb * s.nst_h[k];
+    yx_lines += 4.0 * s.nb * (s.npl_h[k] + n2);
+  }
+  const double c = sizeof(float2), V = (double)s.br_elems() * nv, G = (double)s.rows() * nv * s.nr;
+  const double Gu = (double)s.rows() * s.nr, S1 = nv * st_rows * n3;
+  const double z_fl = nv * st_rows * 5.0 * n3 * std::log2((double)n3);
+  const double yx_fl = nv * yx_lines * n3 * 5.0 * n2 * std::log2((double)n2);
+  const bool density = use_h || use_xc;
+  {
+    ProfScope ps(pf, st, ST_SCATTER, V * c + S1 * c, z_fl);
+    sticks_inverse<float>(ctx, s, x, i1, nv);
+  }
+  {
+    // sticks and U in, x(r) and partial densities out (one kernel: counted as the density's)
+    NvtxRange lines("tdlz/fft_inv");
+    const double nch = slab_density_chunks(s);
+    ProfScope ps(pf, st, density ? ST_DENSITY : ST_FFT_INV,
+                 (S1 + G) * c + (density ? (Gu + (2 * nch + 1) * 4.0 * nv * s.nr) * c : 0.0),
+                 yx_fl + (density ? G / 2 * 40.0 : 0.0));
+    slab_inverse_density(ctx, s, i1, us, d.wk.as<float>(), xs, w.rhopart.as<float2>(), rho, nv,
+                         density);
+  }
+  if (use_h) hartree();
+  {
+    ProfScope ps(pf, st, ST_POTENTIAL, nv * s.nr * (11.0 * c + 14.0 * sizeof(float)),
+                 16.0 * 4 * s.nr * nv);
+    slab_potential(ctx, s, rho, hg, d.fxc.as<float>(), d.vloc.as<float>(),
+                   d.bfield.as<float>(), vp, nv, use_h, use_xc);
+  }
+  {
+    // x(r) and U in, sticks out
+    NvtxRange lines("tdlz/fft_fwd");
+    ProfScope ps(pf, st, ST_PRODUCT, (G + Gu + S1) * c + 6.0 * nv * s.nr * c,
+                 yx_fl + G / 2 * 64.0);
+    slab_product_forward(ctx, s, xs, us, vp, i1, nv);
+  }
+  {
+    ProfScope ps(pf, st, ST_GATHER, S1 * c + 3 * V * c, z_fl);
+    sticks_forward<float>(ctx, s, x, i1, d.kin.as<float>(), d.evals.as<float>(), h, nv);
+  }
+}
+
 template <class T>
 void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nvec,
                        unsigned adj_mask) {
@@ -1352,6 +1410,12 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
       const cx<T> *xs = x + (long long)v0 * br;
       cx<T> *hs = h + (long long)v0 * br;
       const double Gm = (double)s.rows() * m * nr;
+      if constexpr (sizeof(T) == 4) {
+        if (s.slab32) {  // the same steps on plane-ordered grids (slab.cu)
+          slab_stages(ctx, s, d, w, xs, hs, m, use_h, use_xc, [&] { hartree(m); });
+          continue;
+        }
+      }
       // 1. sphere -> real space (pruned Z, Y passes; full X pass)
       pipeline_inverse<T>(ctx, s, xs, xr, i1, i2, m);  // profiled per stage inside
       // 2-4. densities and HXC potentials (one set per vector)
