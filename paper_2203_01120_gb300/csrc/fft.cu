@@ -65,58 +65,18 @@ __device__ __forceinline__ void small_dft(cx<T> *v, int R, int dir, cx<T> w3, cx
   }
 }
 
-// One axis pass.  A tile holds TL lines of length n in shared memory laid out
-// [j][TL+1] (line index fastest, padded) so butterflies on neighbouring lines
-// hit distinct banks.  S == 1: lines are contiguous rows (tile = TL rows);
-// S > 1: lines have stride S and the tile takes TL consecutive inner offsets.
+// Stockham stages on a tile: TL lines of length n in shared memory at in[j (TL + 1) + l];
+// returns the buffer (in or out) that holds the result.
 template <class T, int TL>
-__global__ void __launch_bounds__(256) fft_axis_kernel(cx<T> *__restrict__ data, int n, long long S,
-                                                      long long outer, Stages st,
-                                                      const cx<T> *__restrict__ tw, int dir) {
-  extern __shared__ unsigned char smem_raw[];
+__device__ cx<T> *tile_stages(cx<T> *in, cx<T> *out, int n, const Stages &st, const cx<T> *tw,
+                              int dir) {
   constexpr int P = TL + 1;
-  cx<T> *buf0 = reinterpret_cast<cx<T> *>(smem_raw);
-  cx<T> *buf1 = buf0 + (size_t)n * P;
-  long long tile = blockIdx.x;
-  long long base, jstride, lstride;
-  int nlines;
-  if (S == 1) {
-    long long o0 = tile * TL;
-    long long rem = outer - o0;
-    nlines = rem < TL ? (int)rem : TL;
-    base = o0 * n;
-    jstride = 1;
-    lstride = n;
-  } else {
-    long long tpo = (S + TL - 1) / TL;
-    long long o = tile / tpo;
-    long long i0 = (tile - o * tpo) * TL;
-    long long rem = S - i0;
-    nlines = rem < TL ? (int)rem : TL;
-    base = o * (long long)n * S + i0;
-    jstride = S;
-    lstride = 1;
-  }
-  const int total = n * TL;
-  for (int e = threadIdx.x; e < total; e += blockDim.x) {
-    int j, l;
-    if (S == 1) {
-      l = e / n;
-      j = e - l * n;
-    } else {
-      j = e / TL;
-      l = e - j * TL;
-    }
-    if (l < nlines) buf0[j * P + l] = data[base + j * jstride + l * lstride];
-  }
-  __syncthreads();
   cx<T> w3 = czero<T>(), w5a = czero<T>(), w5b = czero<T>();
   if (n % 3 == 0) w3 = root<T>(tw, n / 3, dir);
   if (n % 5 == 0) {
     w5a = root<T>(tw, n / 5, dir);
     w5b = root<T>(tw, (2 * n) / 5, dir);
   }
-  cx<T> *in = buf0, *out = buf1;
   int ns = 1;
   for (int s = 0; s < st.nrad; ++s) {
     const int R = st.radix[s];
@@ -147,6 +107,79 @@ __global__ void __launch_bounds__(256) fft_axis_kernel(cx<T> *__restrict__ data,
     out = t;
     ns *= R;
   }
+  return in;
+}
+
+// One axis pass.  A tile holds TL lines of length n in shared memory laid out
+// [j][TL+1] (line index fastest, padded) so butterflies on neighbouring lines
+// hit distinct banks.  S == 1: lines are contiguous rows (tile = TL rows);
+// S > 1: lines have stride S and the tile takes TL consecutive inner offsets.
+// MODE 0: in place.  MODE 1 (S == 1): line o is read from
+// src[(o / src_lines) src_stride + (o % src_lines) n].  MODE 2 (one batch per S lines):
+// forward transform, times fac[j S + i], inverse transform.
+enum { AXIS_PLAIN = 0, AXIS_FROM = 1, AXIS_FILTER = 2 };
+template <class T> struct AxisIO {
+  const cx<T> *src;
+  long long src_lines, src_stride;
+  const T *fac;
+};
+template <class T, int TL, int MODE>
+__global__ void __launch_bounds__(256) fft_axis_kernel(cx<T> *__restrict__ data, int n, long long S,
+                                                      long long outer, Stages st,
+                                                      const cx<T> *__restrict__ tw, int dir,
+                                                      AxisIO<T> io) {
+  extern __shared__ unsigned char smem_raw[];
+  constexpr int P = TL + 1;
+  cx<T> *buf0 = reinterpret_cast<cx<T> *>(smem_raw);
+  cx<T> *buf1 = buf0 + (size_t)n * P;
+  long long tile = blockIdx.x;
+  long long base, jstride, lstride, i0 = 0, o0 = 0;
+  int nlines;
+  if (S == 1) {
+    o0 = tile * TL;
+    long long rem = outer - o0;
+    nlines = rem < TL ? (int)rem : TL;
+    base = o0 * n;
+    jstride = 1;
+    lstride = n;
+  } else {
+    long long tpo = (S + TL - 1) / TL;
+    long long o = tile / tpo;
+    i0 = (tile - o * tpo) * TL;
+    long long rem = S - i0;
+    nlines = rem < TL ? (int)rem : TL;
+    base = o * (long long)n * S + i0;
+    jstride = S;
+    lstride = 1;
+  }
+  const int total = n * TL;
+  for (int e = threadIdx.x; e < total; e += blockDim.x) {
+    int j, l;
+    if (S == 1) {
+      l = e / n;
+      j = e - l * n;
+    } else {
+      j = e / TL;
+      l = e - j * TL;
+    }
+    if (l >= nlines) continue;
+    if (MODE == AXIS_FROM) {
+      const long long o = o0 + l, b = o / io.src_lines;
+      buf0[j * P + l] = io.src[b * io.src_stride + (o - b * io.src_lines) * n + j];
+    } else {
+      buf0[j * P + l] = data[base + j * jstride + l * lstride];
+    }
+  }
+  __syncthreads();
+  cx<T> *in = tile_stages<T, TL>(buf0, buf1, n, st, tw, MODE == AXIS_FILTER ? -1 : dir);
+  if (MODE == AXIS_FILTER) {
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+      const int j = e / TL, l = e - j * TL;
+      if (l < nlines) in[j * P + l] = cscale<T>(in[j * P + l], io.fac[j * S + i0 + l]);
+    }
+    __syncthreads();
+    in = tile_stages<T, TL>(in, in == buf0 ? buf1 : buf0, n, st, tw, +1);
+  }
   for (int e = threadIdx.x; e < total; e += blockDim.x) {
     int j, l;
     if (S == 1) {
@@ -167,30 +200,37 @@ Stages stages_of(const AxisPlan &a) {
   return s;
 }
 
-template <class T, int TL>
+long long tiles_of(long long S, long long outer, int tl) {
+  return S == 1 ? (outer + tl - 1) / tl : outer * ((S + tl - 1) / tl);
+}
+
+template <class T, int TL, int MODE>
 void launch_axis(const AxisPlan &a, cx<T> *data, long long S, long long outer, int dir,
-                 cudaStream_t st) {
+                 cudaStream_t st, const AxisIO<T> &io) {
   size_t smem = 2ull * a.n * (TL + 1) * sizeof(cx<T>);
-  long long tiles = (S == 1) ? (outer + TL - 1) / TL : outer * ((S + TL - 1) / TL);
-  TDLZ_CUDA_TRY(cudaFuncSetAttribute(fft_axis_kernel<T, TL>,
+  TDLZ_CUDA_TRY(cudaFuncSetAttribute(fft_axis_kernel<T, TL, MODE>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const cx<T> *tw;
   if constexpr (sizeof(T) == 8)
     tw = a.tw_d;
   else
     tw = a.tw_f;
-  fft_axis_kernel<T, TL><<<(unsigned)tiles, 256, smem, st>>>(data, a.n, S, outer, stages_of(a), tw,
-                                                            dir);
+  fft_axis_kernel<T, TL, MODE><<<(unsigned)tiles_of(S, outer, TL), 256, smem, st>>>(
+      data, a.n, S, outer, stages_of(a), tw, dir, io);
   TDLZ_LAUNCH_CHECK();
 }
 
-template <class T>
+// Lines per tile: 32 (16 above 64 points, shared memory), fewer where that leaves SMs
+// without a tile (one vector of the 16^3 cell: 8 tiles of 32 lines).
+template <class T, int MODE = AXIS_PLAIN>
 void axis_pass(const AxisPlan &a, cx<T> *data, long long S, long long outer, int dir,
-               cudaStream_t st) {
-  if (a.n <= 64)
-    launch_axis<T, 32>(a, data, S, outer, dir, st);
+               cudaStream_t st, const AxisIO<T> &io = AxisIO<T>{}) {
+  if (tiles_of(S, outer, 16) < 152)
+    launch_axis<T, 8, MODE>(a, data, S, outer, dir, st, io);
+  else if (a.n <= 64)
+    launch_axis<T, 32, MODE>(a, data, S, outer, dir, st, io);
   else
-    launch_axis<T, 16>(a, data, S, outer, dir, st);
+    launch_axis<T, 16, MODE>(a, data, S, outer, dir, st, io);
 }
 
 }  // namespace
@@ -252,6 +292,26 @@ void fft3d(const FFTPlan &plan, cx<T> *data, long long batch, int dir, cudaStrea
   axis_pass<T>(plan.ax[0], data, n2 * n3, batch, dir, st);
 }
 
+template <class T>
+void fft3d_filter(const FFTPlan &plan, const cx<T> *src, long long src_stride, const T *fac,
+                  cx<T> *data, long long batch, cudaStream_t st) {
+  const long long n1 = plan.n[0], n2 = plan.n[1], n3 = plan.n[2];
+  AxisIO<T> io{};
+  io.src = src;
+  io.src_lines = n1 * n2;
+  io.src_stride = src_stride;
+  io.fac = fac;
+  axis_pass<T, AXIS_FROM>(plan.ax[2], data, 1, batch * n1 * n2, -1, st, io);
+  axis_pass<T>(plan.ax[1], data, n3, batch * n1, -1, st);
+  axis_pass<T, AXIS_FILTER>(plan.ax[0], data, n2 * n3, batch, 0, st, io);
+  axis_pass<T>(plan.ax[1], data, n3, batch * n1, +1, st);
+  axis_pass<T>(plan.ax[2], data, 1, batch * n1 * n2, +1, st);
+}
+
+template void fft3d_filter<double>(const FFTPlan &, const double2 *, long long, const double *,
+                                   double2 *, long long, cudaStream_t);
+template void fft3d_filter<float>(const FFTPlan &, const float2 *, long long, const float *,
+                                  float2 *, long long, cudaStream_t);
 template void fft3d<double>(const FFTPlan &, double2 *, long long, int, cudaStream_t);
 template void fft3d<float>(const FFTPlan &, float2 *, long long, int, cudaStream_t);
 

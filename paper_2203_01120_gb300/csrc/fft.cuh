@@ -36,4 +36,12 @@ void fft3d(const FFTPlan &plan, cx<T> *data, long long batch, int dir, cudaStrea
 
 bool fft_length_supported(int n);
 
+// data[b] = IFFT(fac x FFT(src[b])) for batch b = 0..batch-1: unnormalised transforms, source
+// grids src_stride elements apart, the same real factors fac[Nr] for every batch.  Five axis
+// passes: the first reads the source, the first axis runs its forward transform, the factors
+// and its inverse transform on the tile in shared memory.
+template <class T>
+void fft3d_filter(const FFTPlan &plan, const cx<T> *src, long long src_stride, const T *fac,
+                  cx<T> *data, long long batch, cudaStream_t st);
+
 }  // namespace tdlz

@@ -23,6 +23,7 @@
 //  PHM  metric M = J L (positive definite when D + K > 0): alpha = (Lq)^H J (Lq);
 //       r = Lq - alpha q - beta q'; w = L r; c = r^H J w; beta' = sqrt c;
 //       q = r/beta', Lq = w/beta' (the product of the step is the one on r).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -51,25 +52,48 @@ struct Pairs {
 constexpr int kPStride = 5;
 
 
+// Up to four chains of a group handled by one launch (block row or block = chain).
+constexpr int kStepChains = 4;
+constexpr long long kPartials = (long long)kRedBlocks * kPStride;  // of one chain
+struct StepArgs {
+  const void *a[kStepChains], *q[kStepChains], *b[kStepChains], *p[kStepChains];
+  void *qp[kStepChains], *pp[kStepChains];
+  ChainScalars *cs[kStepChains];
+  ChainCoeffs cf[kStepChains];
+};
+struct PairSet {
+  Pairs c[kStepChains];
+};
+
 // Block-level deterministic sum of NV complex values per thread into
-// out[blockIdx][0..NV) (row stride kPStride).
+// out[blockIdx.x][0..NV) (row stride kPStride).  The values go down the tree together: its
+// eight levels of FP64 sums and barriers are paid once, not per value.
 template <int NV>
 __device__ void block_sum_store(double2 (&v)[NV], double2 *out) {
   static_assert(NV <= kPStride, "partial row");
-  __shared__ double2 sh[kRedThreads];
-  for (int q = 0; q < NV; ++q) {
-    sh[threadIdx.x] = v[q];
-    __syncthreads();
-    for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-      if (threadIdx.x < s) {
-        sh[threadIdx.x].x += sh[threadIdx.x + s].x;
-        sh[threadIdx.x].y += sh[threadIdx.x + s].y;
+  __shared__ double2 sh[NV][kRedThreads];
+#pragma unroll
+  for (int q = 0; q < NV; ++q) sh[q][threadIdx.x] = v[q];
+  __syncthreads();
+  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
+    if (threadIdx.x < s) {
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        sh[q][threadIdx.x].x += sh[q][threadIdx.x + s].x;
+        sh[q][threadIdx.x].y += sh[q][threadIdx.x + s].y;
       }
-      __syncthreads();
     }
-    if (threadIdx.x == 0) out[(long long)blockIdx.x * kPStride + q] = sh[0];
     __syncthreads();
   }
+  if (threadIdx.x < NV) out[(long long)blockIdx.x * kPStride + threadIdx.x] = sh[threadIdx.x][0];
+  __syncthreads();
+}
+
+// Blocks of a reduction over n elements: one element per thread for short vectors (a block
+// of an idle SM costs nothing, and the fixed 1024 blocks' tails cost 134 us per step of the
+// 16^3 cell's 9760 elements), at most kRedBlocks.
+inline int red_blocks(long long n) {
+  return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + kRedThreads - 1) / kRedThreads));
 }
 
 // partial[blk][i] = sum_{e in blk range} conj(a_i[e]) b_i[e] (J-weighted if requested)
@@ -81,7 +105,9 @@ constexpr int kRun = 16;
 constexpr int kUnroll = 4;  // independent elements per thread per iteration (loads in flight)
 template <class T, int NP>
 __global__ void __launch_bounds__(kRedThreads)
-    dots_kernel(Pairs pr, long long n, long long half, double2 *partial) {
+    dots_kernel(PairSet ps, long long n, long long half, double2 *partial) {
+  const Pairs &pr = ps.c[blockIdx.y];
+  partial += blockIdx.y * kPartials;
   double2 acc[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) acc[i] = make_double2(0.0, 0.0);
@@ -134,35 +160,39 @@ __global__ void __launch_bounds__(kRedThreads)
   block_sum_store<NP>(acc, partial);
 }
 
-// Sum the partials of nv values in fixed order; result into out[nv].
+// Sum the partials of nv <= kPStride values in fixed order; result into out[nv].
 __device__ void reduce_partials(const double2 *partial, int nblk, int nv, double2 *out) {
-  __shared__ double2 sh[kRedThreads];
+  __shared__ double2 sh[kPStride][kRedThreads];
   for (int q = 0; q < nv; ++q) {
     double2 s = {0, 0};
     for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
       s.x += partial[(long long)b * kPStride + q].x;
       s.y += partial[(long long)b * kPStride + q].y;
     }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int st = kRedThreads / 2; st > 0; st >>= 1) {
-      if (threadIdx.x < st) {
-        sh[threadIdx.x].x += sh[threadIdx.x + st].x;
-        sh[threadIdx.x].y += sh[threadIdx.x + st].y;
+    sh[q][threadIdx.x] = s;
+  }
+  __syncthreads();
+  for (int st = kRedThreads / 2; st > 0; st >>= 1) {
+    if (threadIdx.x < st)
+      for (int q = 0; q < nv; ++q) {
+        sh[q][threadIdx.x].x += sh[q][threadIdx.x + st].x;
+        sh[q][threadIdx.x].y += sh[q][threadIdx.x + st].y;
       }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[q] = sh[0];
     __syncthreads();
   }
+  if (threadIdx.x < nv) out[threadIdx.x] = sh[threadIdx.x][0];
+  __syncthreads();
 }
 
 __device__ __forceinline__ bool finite2(double2 v) { return isfinite(v.x) && isfinite(v.y); }
 
 // ---------------------------------------------------------------- scalars
 // Stage A: alpha and z from the dots (d0 = alpha source, d1..nz = q^H u^l).
-__global__ void scalar_a_kernel(const double2 *partial, int nblk, ChainScalars *cs,
-                                ChainCoeffs cf, int flavor, int nz) {
+__global__ void scalar_a_kernel(const double2 *partial, int nblk, StepArgs sa, int flavor,
+                                int nz) {
+  ChainScalars *cs = sa.cs[blockIdx.x];
+  const ChainCoeffs &cf = sa.cf[blockIdx.x];
+  partial += blockIdx.x * kPartials;
   __shared__ double2 d[kPStride];
   reduce_partials(partial, nblk, 1 + nz, d);
   if (threadIdx.x != 0) return;
@@ -190,8 +220,10 @@ __global__ void scalar_a_kernel(const double2 *partial, int nblk, ChainScalars *
 }
 
 // Stage B: beta, gamma, signs and rescale factors from c (d0) and norms (d1, d2).
-__global__ void scalar_b_kernel(const double2 *partial, int nblk, ChainScalars *cs,
-                                ChainCoeffs cf, int flavor) {
+__global__ void scalar_b_kernel(const double2 *partial, int nblk, StepArgs sa, int flavor) {
+  ChainScalars *cs = sa.cs[blockIdx.x];
+  const ChainCoeffs &cf = sa.cf[blockIdx.x];
+  partial += blockIdx.x * kPartials;
   __shared__ double2 d[kPStride];
   reduce_partials(partial, nblk, 3, d);
   if (threadIdx.x != 0) return;
@@ -317,9 +349,15 @@ __global__ void scale_kernel(cx<T> *x, const double2 *scale, long long n) {
 // (r, r), (t~, t~) = (t, t).
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-    update_kernel(const cx<T> *a, const cx<T> *q, cx<T> *qp, const cx<T> *b, const cx<T> *p,
-                  cx<T> *pp, const ChainScalars *cs, int flavor, long long n, long long half,
-                  double2 *partial) {
+    update_kernel(StepArgs sa, int flavor, long long n, long long half, double2 *partial) {
+  const int ch = blockIdx.y;
+  const cx<T> *a = reinterpret_cast<const cx<T> *>(sa.a[ch]);
+  const cx<T> *q = reinterpret_cast<const cx<T> *>(sa.q[ch]);
+  const cx<T> *b = reinterpret_cast<const cx<T> *>(sa.b[ch]);
+  const cx<T> *p = reinterpret_cast<const cx<T> *>(sa.p[ch]);
+  cx<T> *qp = reinterpret_cast<cx<T> *>(sa.qp[ch]), *pp = reinterpret_cast<cx<T> *>(sa.pp[ch]);
+  const ChainScalars *cs = sa.cs[ch];
+  partial += ch * kPartials;
   // coefficients in the vectors' precision (FP64 path: exact; mixed: rounded to FP32,
   // an error of the order of the FP32 storage of r itself)
   const double2 a64 = cs->alpha;
@@ -452,7 +490,7 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 #pragma unroll
   for (int c = 0; c < M; ++c)
-    block_sum_store<NA>(acc[c], partial + (long long)c * gridDim.x * kPStride);
+    block_sum_store<NA>(acc[c], partial + c * kPartials);
 }
 
 // x_v *= *s_v for the nv vectors of a set (the new Lanczos vectors of a group)
@@ -482,14 +520,17 @@ __global__ void jflip_kernel(const cx<T> *x, cx<T> *y, long long n, long long ha
   }
 }
 
+// Dots of m <= kStepChains chains (the same number of pairs each).
 template <class T>
-void launch_dots(Context &ctx, Pairs pr, long long n, long long half, double2 *partial) {
-  switch (pr.n) {
-    case 1: dots_kernel<T, 1><<<kRedBlocks, kRedThreads, 0, ctx.stream>>>(pr, n, half, partial); break;
-    case 2: dots_kernel<T, 2><<<kRedBlocks, kRedThreads, 0, ctx.stream>>>(pr, n, half, partial); break;
-    case 3: dots_kernel<T, 3><<<kRedBlocks, kRedThreads, 0, ctx.stream>>>(pr, n, half, partial); break;
-    case 4: dots_kernel<T, 4><<<kRedBlocks, kRedThreads, 0, ctx.stream>>>(pr, n, half, partial); break;
-    default: dots_kernel<T, 5><<<kRedBlocks, kRedThreads, 0, ctx.stream>>>(pr, n, half, partial); break;
+void launch_dots(Context &ctx, const PairSet &ps, int m, long long n, long long half,
+                 double2 *partial) {
+  const dim3 g(red_blocks(n), m);
+  switch (ps.c[0].n) {
+    case 1: dots_kernel<T, 1><<<g, kRedThreads, 0, ctx.stream>>>(ps, n, half, partial); break;
+    case 2: dots_kernel<T, 2><<<g, kRedThreads, 0, ctx.stream>>>(ps, n, half, partial); break;
+    case 3: dots_kernel<T, 3><<<g, kRedThreads, 0, ctx.stream>>>(ps, n, half, partial); break;
+    case 4: dots_kernel<T, 4><<<g, kRedThreads, 0, ctx.stream>>>(ps, n, half, partial); break;
+    default: dots_kernel<T, 5><<<g, kRedThreads, 0, ctx.stream>>>(ps, n, half, partial); break;
   }
   TDLZ_LAUNCH_CHECK();
 }
@@ -515,7 +556,7 @@ template void jflip_copy<float>(Context &, QSlot &, const float2 *, float2 *);
 template <class T>
 void ChainSet::init_impl() {
   const size_t c = sizeof(cx<T>);
-  red.alloc((size_t)kRedBlocks * kPStride * 16 * sizeof(double2));  // up to 16 chains per group
+  red.alloc((size_t)kPartials * kStepChains * sizeof(double2));
   for (size_t i = 0; i < chains.size(); ++i) {
     Chain &ch = chains[i];
     int g = -1;
@@ -560,14 +601,14 @@ void ChainSet::init_impl() {
       Chain &ch = chains[gr.members[mi]];
       ChainScalars *cs = ch.sc.as<ChainScalars>();
       cx<T> *Q = (cx<T> *)gr.slot[0] + mi * n;
-      Pairs pr{};
-      pr.n = 1;
+      PairSet ps{};
+      ps.c[0].n = 1;
       if (flavor == TDLZ_PSEUDOHERMITIAN_POSDEF)
-        pr.p[0] = Pair{Q, (cx<T> *)gr.slot[3] + mi * n, 1};
+        ps.c[0].p[0] = Pair{Q, (cx<T> *)gr.slot[3] + mi * n, 1};
       else
-        pr.p[0] = Pair{Q, Q, flavor == TDLZ_PSEUDOHERMITIAN ? 1 : 0};
-      launch_dots<T>(*ctx, pr, n, half, part);
-      scalar_init_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, flavor);
+        ps.c[0].p[0] = Pair{Q, Q, flavor == TDLZ_PSEUDOHERMITIAN ? 1 : 0};
+      launch_dots<T>(*ctx, ps, 1, n, half, part);
+      scalar_init_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, red_blocks(n), cs, flavor);
       TDLZ_LAUNCH_CHECK();
       scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(Q, &cs->scale_q, n);
       TDLZ_LAUNCH_CHECK();
@@ -586,35 +627,64 @@ void ChainSet::init_impl() {
 template <class T>
 void ChainSet::advance_impl(int nsteps) {
   double2 *part = red.as<double2>();
+  cudaStream_t st = ctx->stream;
   for (int it = 0; it < nsteps; ++it) {
     for (Group &gr : groups) {
       if (gr.host_step >= cap) continue;
       QSlot &s = *ctx->slots[gr.qslot];
       const long long n = s.br_elems(), half = n / 2;
-      const int m = (int)gr.members.size();
+      const int m = (int)gr.members.size(), nblk = red_blocks(n);
       const cx<T> *u = slot_data<T>(s).uvec.template as<cx<T>>();
       cx<T> *S0 = (cx<T> *)gr.slot[0], *S1 = (cx<T> *)gr.slot[1], *S2 = (cx<T> *)gr.slot[2];
-      if (flavor == TDLZ_NONHERMITIAN) {
-        // a = L q and b~ = L p~ = J L^H p for every member in one pass
-        apply_liouvillian<T>(*ctx, s, S0, S2, 2 * m, 0u);
-        if (m <= 4) {
-          // the group's dots in one pass (u^l read once), then per chain the scalars and
-          // the update, then every new vector rescaled in one launch
-          ProfScope ps(ctx->prof, ctx->stream, ST_LANCZOS, (15.0 * m + 3.0) * n * sizeof(cx<T>),
-                       40.0 * m * n);
+      cx<T> *S3 = (cx<T> *)gr.slot[3];
+      const bool nh = flavor == TDLZ_NONHERMITIAN, phm = flavor == TDLZ_PSEUDOHERMITIAN_POSDEF;
+      // NH: a = L q and b~ = L p~ = J L^H p for every member in one pass; PH: a = L q
+      if (!phm) apply_liouvillian<T>(*ctx, s, S0, S2, nh ? 2 * m : m, 0u);
+      // Chains m0 .. m0 + mc - 1 share each launch: their dots (NH reads every u^l once),
+      // the scalars alpha and z, the three-term update with the new residual's dots, the
+      // scalars beta and gamma, and the new vectors' rescaling.
+      for (int m0 = 0; m0 < m; m0 += kStepChains) {
+        const int mc = std::min(kStepChains, m - m0);
+        StepArgs sa{};
+        ScaleSet ss{};
+        for (int i = 0; i < mc; ++i) {
+          const long long o = (m0 + i) * n, op = (m + m0 + i) * n;
+          Chain &ch = chains[gr.members[m0 + i]];
+          ChainScalars *cs = ch.sc.as<ChainScalars>();
+          sa.a[i] = S2 + o;
+          sa.q[i] = S0 + o;
+          sa.qp[i] = S1 + o;
+          if (nh) {
+            sa.b[i] = S2 + op;
+            sa.p[i] = S0 + op;
+            sa.pp[i] = S1 + op;
+          }
+          sa.cs[i] = cs;
+          sa.cf[i] = ch.cf;
+          ss.x[i] = S1 + o;
+          ss.s[i] = &cs->scale_q;
+          if (nh) {
+            ss.x[mc + i] = S1 + op;
+            ss.s[mc + i] = &cs->scale_p;
+          }
+        }
+        ProfScope ps(ctx->prof, st, ST_LANCZOS,
+                     ((nh ? 15.0 : phm ? 9.0 : 11.0) * mc + (nh ? 3.0 : 0.0)) * n * sizeof(cx<T>),
+                     (nh ? 40.0 : 28.0) * mc * n);
+        if (nh) {
           NhGroupDots gd{};
-          for (int mi = 0; mi < m; ++mi) {
-            gd.q[mi] = S0 + mi * n;
-            gd.p[mi] = S0 + (m + mi) * n;
-            gd.a[mi] = S2 + mi * n;
+          for (int i = 0; i < mc; ++i) {
+            gd.q[i] = sa.q[i];
+            gd.p[i] = sa.p[i];
+            gd.a[i] = sa.a[i];
           }
           for (int l = 0; l < ncomp; ++l) gd.u[l] = u + l * n;
-#define TDLZ_NH_DOTS(MM)                                                                   \
-  if (ncomp == 4)                                                                           \
-    nh_group_dots_kernel<T, MM, 4><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(gd, n, half, part); \
-  else                                                                                      \
-    nh_group_dots_kernel<T, MM, 3><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(gd, n, half, part);
-          switch (m) {
+#define TDLZ_NH_DOTS(MM)                                                          \
+  if (ncomp == 4)                                                                  \
+    nh_group_dots_kernel<T, MM, 4><<<nblk, kRedThreads, 0, st>>>(gd, n, half, part); \
+  else                                                                             \
+    nh_group_dots_kernel<T, MM, 3><<<nblk, kRedThreads, 0, st>>>(gd, n, half, part);
+          switch (mc) {
             case 1: TDLZ_NH_DOTS(1) break;
             case 2: TDLZ_NH_DOTS(2) break;
             case 3: TDLZ_NH_DOTS(3) break;
@@ -622,131 +692,57 @@ void ChainSet::advance_impl(int nsteps) {
           }
 #undef TDLZ_NH_DOTS
           TDLZ_LAUNCH_CHECK();
-          const long long pstride = (long long)kRedBlocks * kPStride;
-          for (int mi = 0; mi < m; ++mi) {
-            Chain &ch = chains[gr.members[mi]];
-            scalar_a_kernel<<<1, kRedThreads, 0, ctx->stream>>>(
-                part + mi * pstride, kRedBlocks, ch.sc.as<ChainScalars>(), ch.cf, flavor, ncomp);
-            TDLZ_LAUNCH_CHECK();
+        } else {
+          PairSet pr{};
+          for (int i = 0; i < mc; ++i) {
+            pr.c[i].n = 1 + ncomp;
+            pr.c[i].p[0] = phm ? Pair{sa.a[i], sa.a[i], 1} : Pair{sa.q[i], sa.a[i], 1};
+            for (int l = 0; l < ncomp; ++l) pr.c[i].p[1 + l] = Pair{sa.q[i], u + l * n, 0};
           }
-          ScaleSet ss{};
-          for (int mi = 0; mi < m; ++mi) {
-            Chain &ch = chains[gr.members[mi]];
-            ChainScalars *cs = ch.sc.as<ChainScalars>();
-            cx<T> *Q = S0 + mi * n, *P = S0 + (m + mi) * n, *QP = S1 + mi * n,
-                  *PP = S1 + (m + mi) * n, *A = S2 + mi * n, *B = S2 + (m + mi) * n;
-            double2 *pc = part + mi * pstride;
-            update_kernel<T><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(A, Q, QP, B, P, PP, cs,
-                                                                         flavor, n, half, pc);
-            TDLZ_LAUNCH_CHECK();
-            scalar_b_kernel<<<1, kRedThreads, 0, ctx->stream>>>(pc, kRedBlocks, cs, ch.cf, flavor);
-            TDLZ_LAUNCH_CHECK();
-            ss.x[mi] = QP;
-            ss.s[mi] = &cs->scale_q;
-            ss.x[m + mi] = PP;
-            ss.s[m + mi] = &cs->scale_p;
-          }
-          scale_set_kernel<T><<<dim3(blocks_for(n) / 2 + 1, 2 * m), 256, 0, ctx->stream>>>(ss, n);
-          TDLZ_LAUNCH_CHECK();
-          std::swap(gr.slot[0], gr.slot[1]);
-          gr.host_step++;
-          continue;
+          launch_dots<T>(*ctx, pr, mc, n, half, part);
         }
-        ProfScope ps(ctx->prof, ctx->stream, ST_LANCZOS, 18.0 * m * n * sizeof(cx<T>),
-                     40.0 * m * n);
-        for (int mi = 0; mi < m; ++mi) {
-          Chain &ch = chains[gr.members[mi]];
-          ChainScalars *cs = ch.sc.as<ChainScalars>();
-          cx<T> *Q = S0 + mi * n, *P = S0 + (m + mi) * n, *QP = S1 + mi * n,
-                *PP = S1 + (m + mi) * n, *A = S2 + mi * n, *B = S2 + (m + mi) * n;
-          Pairs pr{};
-          pr.n = 1 + ncomp;
-          pr.p[0] = Pair{P, A, 1};  // p^H a = p~^H J a
-          for (int l = 0; l < ncomp; ++l) pr.p[1 + l] = Pair{Q, u + l * n, 0};
-          launch_dots<T>(*ctx, pr, n, half, part);
-          scalar_a_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf, flavor,
-                                                              ncomp);
-          TDLZ_LAUNCH_CHECK();
-          update_kernel<T><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(A, Q, QP, B, P, PP, cs,
-                                                                       flavor, n, half, part);
-          TDLZ_LAUNCH_CHECK();
-          scalar_b_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf, flavor);
-          TDLZ_LAUNCH_CHECK();
-          scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(QP, &cs->scale_q, n);
-          scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(PP, &cs->scale_p, n);
-          TDLZ_LAUNCH_CHECK();
-        }
-        std::swap(gr.slot[0], gr.slot[1]);
-      } else if (flavor == TDLZ_PSEUDOHERMITIAN) {
-        apply_liouvillian<T>(*ctx, s, S0, S2, m, 0u);
-        ProfScope ps(ctx->prof, ctx->stream, ST_LANCZOS, 11.0 * m * n * sizeof(cx<T>),
-                     28.0 * m * n);
-        for (int mi = 0; mi < m; ++mi) {
-          Chain &ch = chains[gr.members[mi]];
-          ChainScalars *cs = ch.sc.as<ChainScalars>();
-          cx<T> *Q = S0 + mi * n, *QP = S1 + mi * n, *A = S2 + mi * n;
-          Pairs pr{};
-          pr.n = 1 + ncomp;
-          pr.p[0] = Pair{Q, A, 1};
-          for (int l = 0; l < ncomp; ++l) pr.p[1 + l] = Pair{Q, u + l * n, 0};
-          launch_dots<T>(*ctx, pr, n, half, part);
-          scalar_a_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf, flavor,
-                                                              ncomp);
-          TDLZ_LAUNCH_CHECK();
-          update_kernel<T><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(
-              A, Q, QP, nullptr, nullptr, nullptr, cs, flavor, n, half, part);
-          TDLZ_LAUNCH_CHECK();
-          scalar_b_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf, flavor);
-          TDLZ_LAUNCH_CHECK();
-          scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(QP, &cs->scale_q, n);
-          TDLZ_LAUNCH_CHECK();
-        }
-        std::swap(gr.slot[0], gr.slot[1]);
-      } else {
-        cx<T> *S3 = (cx<T> *)gr.slot[3];
-        {
-          ProfScope ps(ctx->prof, ctx->stream, ST_LANCZOS, 9.0 * m * n * sizeof(cx<T>),
-                       24.0 * m * n);
-          for (int mi = 0; mi < m; ++mi) {
-            Chain &ch = chains[gr.members[mi]];
-            ChainScalars *cs = ch.sc.as<ChainScalars>();
-            cx<T> *Q = S0 + mi * n, *QP = S1 + mi * n, *LQ = S2 + mi * n;
-            Pairs pr{};
-            pr.n = 1 + ncomp;
-            pr.p[0] = Pair{LQ, LQ, 1};
-            for (int l = 0; l < ncomp; ++l) pr.p[1 + l] = Pair{Q, u + l * n, 0};
-            launch_dots<T>(*ctx, pr, n, half, part);
-            scalar_a_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf,
-                                                                flavor, ncomp);
-            TDLZ_LAUNCH_CHECK();
-            update_kernel<T><<<kRedBlocks, kRedThreads, 0, ctx->stream>>>(
-                LQ, Q, QP, nullptr, nullptr, nullptr, cs, flavor, n, half, part);
-            TDLZ_LAUNCH_CHECK();
-          }
-        }
+        scalar_a_kernel<<<mc, kRedThreads, 0, st>>>(part, nblk, sa, flavor, ncomp);
+        TDLZ_LAUNCH_CHECK();
+        update_kernel<T><<<dim3(nblk, mc), kRedThreads, 0, st>>>(sa, flavor, n, half, part);
+        TDLZ_LAUNCH_CHECK();
+        if (phm) continue;  // its residual's dots need w = L r
+        scalar_b_kernel<<<mc, kRedThreads, 0, st>>>(part, nblk, sa, flavor);
+        TDLZ_LAUNCH_CHECK();
+        scale_set_kernel<T><<<dim3(blocks_for(n) / 2 + 1, nh ? 2 * mc : mc), 256, 0, st>>>(ss, n);
+        TDLZ_LAUNCH_CHECK();
+      }
+      if (phm) {
         apply_liouvillian<T>(*ctx, s, S1, S3, m, 0u);  // w = L r for every member
-        ProfScope ps(ctx->prof, ctx->stream, ST_LANCZOS, 6.0 * m * n * sizeof(cx<T>),
-                     12.0 * m * n);
-        for (int mi = 0; mi < m; ++mi) {
-          Chain &ch = chains[gr.members[mi]];
-          ChainScalars *cs = ch.sc.as<ChainScalars>();
-          cx<T> *QP = S1 + mi * n, *W = S3 + mi * n;
-          Pairs pc{};
-          pc.n = 3;
-          pc.p[0] = Pair{QP, W, 1};
-          pc.p[1] = Pair{QP, QP, 0};
-          pc.p[2] = Pair{W, W, 0};
-          launch_dots<T>(*ctx, pc, n, half, part);
-          scalar_b_kernel<<<1, kRedThreads, 0, ctx->stream>>>(part, kRedBlocks, cs, ch.cf, flavor);
+        for (int m0 = 0; m0 < m; m0 += kStepChains) {
+          const int mc = std::min(kStepChains, m - m0);
+          StepArgs sa{};
+          ScaleSet ss{};
+          PairSet pc{};
+          for (int i = 0; i < mc; ++i) {
+            Chain &ch = chains[gr.members[m0 + i]];
+            ChainScalars *cs = ch.sc.as<ChainScalars>();
+            cx<T> *R = S1 + (m0 + i) * n, *W = S3 + (m0 + i) * n;
+            sa.cs[i] = cs;
+            sa.cf[i] = ch.cf;
+            pc.c[i].n = 3;
+            pc.c[i].p[0] = Pair{R, W, 1};
+            pc.c[i].p[1] = Pair{R, R, 0};
+            pc.c[i].p[2] = Pair{W, W, 0};
+            ss.x[i] = R;
+            ss.x[mc + i] = W;
+            ss.s[i] = ss.s[mc + i] = &cs->scale_q;
+          }
+          ProfScope ps(ctx->prof, st, ST_LANCZOS, 6.0 * mc * n * sizeof(cx<T>), 12.0 * mc * n);
+          launch_dots<T>(*ctx, pc, mc, n, half, part);
+          scalar_b_kernel<<<mc, kRedThreads, 0, st>>>(part, nblk, sa, flavor);
           TDLZ_LAUNCH_CHECK();
-          scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(QP, &cs->scale_q, n);
-          scale_kernel<T><<<blocks_for(n), 256, 0, ctx->stream>>>(W, &cs->scale_q, n);
+          scale_set_kernel<T><<<dim3(blocks_for(n) / 2 + 1, 2 * mc), 256, 0, st>>>(ss, n);
           TDLZ_LAUNCH_CHECK();
         }
-        // q' <- q, q <- r/beta, Lq <- w/beta, w <- old Lq
-        std::swap(gr.slot[0], gr.slot[1]);
+        // Lq <- w/beta, w <- old Lq
         std::swap(gr.slot[2], gr.slot[3]);
       }
+      std::swap(gr.slot[0], gr.slot[1]);  // q' <- q, q <- r/beta
       gr.host_step++;
     }
   }

@@ -799,26 +799,6 @@ void alloc_workspace(QSlot &s, int nvec) {
   w.ready = true;
 }
 
-// a[i] *= fac[i % n] (the Hartree factor of one grid applied to stacked grids)
-template <class T>
-__global__ void scale_periodic_kernel(cx<T> *__restrict__ a, const T *__restrict__ fac,
-                                      long long n, long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x)
-    a[i] = cscale<T>(a[i], fac[i % n]);
-}
-
-// b[v][i] = a[v][stride][i]  (component 0 of each vector's 4-component density)
-template <class T>
-__global__ void gather_component_kernel(const cx<T> *__restrict__ a, cx<T> *__restrict__ b,
-                                        long long n, long long stride, long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    long long v = i / n;
-    b[i] = a[v * stride + (i - v * n)];
-  }
-}
-
 }  // namespace
 
 // ===================================================================== load
@@ -1342,16 +1322,9 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
   const bool use_h = s.kernel_mask & TDLZ_KERNEL_HARTREE, use_xc = s.kernel_mask & TDLZ_KERNEL_XC;
   // Hartree at q (Eq. v_H_q): rho'_0 -> G, 4 pi / |q+G|^2 on the density sphere, -> r
   auto hartree = [&](int nv) {
-    ProfScope ps(pf, st, ST_HARTREE, 8.0 * nv * nr * c,
+    ProfScope ps(pf, st, ST_HARTREE, 11.0 * nv * nr * c,
                  2 * 5.0 * nv * nr * std::log2((double)nr));
-    long long tot = (long long)nv * nr;
-    gather_component_kernel<T><<<blocks_for(tot), kThreads, 0, st>>>(rho, hg, nr, 4 * nr, tot);
-    TDLZ_LAUNCH_CHECK();
-    fft3d<T>(s.plan, hg, nv, -1, st);
-    scale_periodic_kernel<T><<<blocks_for(tot), kThreads, 0, st>>>(
-        hg, d.vhfac.template as<T>(), nr, tot);
-    TDLZ_LAUNCH_CHECK();
-    fft3d<T>(s.plan, hg, nv, +1, st);
+    fft3d_filter<T>(s.plan, rho, 4 * nr, d.vhfac.template as<T>(), hg, nv, st);
   };
   const bool planes = sizeof(T) == 4 ? s.planes32 : s.planes64;
   if (planes) {
