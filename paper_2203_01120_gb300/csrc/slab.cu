@@ -43,6 +43,8 @@ template <int N> struct Slab {
   // with eight warps, forward 8.7 ms against 9.4 with six)
   static constexpr int FTH = N <= 12 ? 96 : N <= 16 ? 128 : N <= 24 ? 192 : 256;
   static constexpr int ITH = N >= 45 ? 192 : FTH;
+  static constexpr int CTAS = N >= 24 ? 2 : 4;  // three of 24 points spill: 0.33 for 0.21 ms
+  static constexpr int PU = N >= 45 ? 4 : 2;    // points a forward thread loads at a time
   static constexpr int P = N + 1;                           // row pitch of a tile
   static constexpr int TROW = N * P;                        // elements of one row's tile
   static constexpr int TILE = 2 * NBS * TROW;
@@ -68,13 +70,21 @@ struct SlabTab {
   long long nnp;
 };
 
-// Walks the groups [g0, g1) of a chunk: pair = side nk + k, first band of the group.
+// Walks the groups [g0, g1) of a chunk: pair = side nk + k, first band of the group, and the
+// pair's sphere: planes, sticks and this thread's first stick's position (read once per pair).
 struct Walk {
-  int pair, n, k;
+  int pair, n, k, ns, pos0;
+  int2 pl;
   __device__ Walk(const SlabTab &tb, int g, int nbs) {
     pair = g / tb.gpp;
     n = (g - pair * tb.gpp) * nbs;
     k = pair % tb.nk;
+    sphere(tb);
+  }
+  __device__ void sphere(const SlabTab &tb) {
+    ns = __ldg(tb.nst + k);
+    pl = __ldg(tb.pl + k);
+    pos0 = (int)threadIdx.x < ns ? __ldg(tb.pos + (long long)k * tb.nsm + threadIdx.x) : 0;
   }
   __device__ void next(const SlabTab &tb, int nbs) {
     n += nbs;
@@ -82,7 +92,12 @@ struct Walk {
       n = 0;
       ++pair;
       if (++k == tb.nk) k = 0;
+      if (pair < 2 * tb.nk) sphere(tb);
     }
+  }
+  // position of stick i = threadIdx.x + j blockDim.x
+  __device__ int pos(const SlabTab &tb, int i) const {
+    return i == (int)threadIdx.x ? pos0 : __ldg(tb.pos + (long long)k * tb.nsm + i);
   }
 };
 
@@ -96,12 +111,12 @@ struct Walk {
 // pot[v][z][3][NN]: (w00, w11), (w01, w10), (h0, h1, B_x, -B_y) of side X; side Y exchanges
 // the first two pairs' members and signs (see product).
 template <int N>
-__global__ void __launch_bounds__(Slab<N>::FTH, 2)
+__global__ void __launch_bounds__(Slab<N>::FTH, Slab<N>::CTAS)
     slab_forward_kernel(const float2 *__restrict__ xs, const float2 *__restrict__ us,
                         const float4 *__restrict__ pot, float2 *__restrict__ i1t, SlabTab tb,
                         int nvec, int glen, const RegTw<float, N> tw) {
   using D = Slab<N>;
-  constexpr int NBS = D::NBS, P = D::P, NN = N * N, TH = D::FTH, PU = 2;
+  constexpr int NBS = D::NBS, P = D::P, NN = N * N, TH = D::FTH, PU = D::PU;
   extern __shared__ float4 slab_smem[];
   float2 *t = reinterpret_cast<float2 *>(slab_smem);  // [2 NBS][N][P]
   const int v = blockIdx.x % nvec, z = blockIdx.y;    // vectors fastest: they share U in L2
@@ -183,7 +198,7 @@ __global__ void __launch_bounds__(Slab<N>::FTH, 2)
         product(std::true_type{});
     }
     __syncthreads();
-    const int2 pl = __ldg(tb.pl + wk.k);
+    const int2 pl = wk.pl;
     if (xr < rows) {
       float2 *c = t + xr * D::TROW + xj;
       float2 a[N];
@@ -211,11 +226,9 @@ __global__ void __launch_bounds__(Slab<N>::FTH, 2)
     }
     __syncthreads();
     {
-      const int ns = __ldg(tb.nst + wk.k);
-      const int *pos = tb.pos + (long long)wk.k * tb.nsm;
       float2 *o = i1t + ((vrow + row0) * tb.n3 + z) * tb.nsm;
-      for (int i = ft; i < ns; i += TH) {
-        const float2 *c = t + __ldg(pos + i);
+      for (int i = ft; i < wk.ns; i += TH) {
+        const float2 *c = t + wk.pos(tb, i);
 #pragma unroll
         for (int r = 0; r < 2 * NBS; ++r)
           if (r < rows) o[(long long)r * tb.n3 * tb.nsm + i] = c[r * D::TROW];
@@ -232,7 +245,7 @@ __global__ void __launch_bounds__(Slab<N>::FTH, 2)
 // Dense stick rows d[2 NBS][npm][P] (zeros where a plane has no stick) follow the tile; the
 // next group's sticks are copied into them (cp.async) while this group's X lines run.
 template <int N, bool DENS>
-__global__ void __launch_bounds__(Slab<N>::ITH, 2)
+__global__ void __launch_bounds__(Slab<N>::ITH, Slab<N>::CTAS)
     slab_inverse_kernel(const float2 *__restrict__ i1t, const float2 *__restrict__ us,
                         const float *__restrict__ wk_, float2 *__restrict__ xs,
                         float2 *__restrict__ part, SlabTab tb, int nvec, int glen,
@@ -269,12 +282,11 @@ __global__ void __launch_bounds__(Slab<N>::ITH, 2)
     }
   };
   auto stage = [&](const Walk &w) {
-    const int rows = 2 * min(NBS, tb.nb - w.n), ns = __ldg(tb.nst + w.k);
+    const int rows = 2 * min(NBS, tb.nb - w.n);
     const long long row0 = vrow + 2LL * ((long long)w.pair * tb.nb + w.n);
-    const int *pos = tb.pos + (long long)w.k * tb.nsm;
     const float2 *src = i1t + (row0 * tb.n3 + z) * tb.nsm;
-    for (int i = ft; i < ns; i += TH) {
-      float2 *o = d + __ldg(pos + i);
+    for (int i = ft; i < w.ns; i += TH) {
+      float2 *o = d + w.pos(tb, i);
 #pragma unroll
       for (int r = 0; r < 2 * NBS; ++r)
         if (r < rows) cp_async8(o + r * drow, src + (long long)r * tb.n3 * tb.nsm + i);
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(Slab<N>::ITH, 2)
     const int nbg = min(NBS, tb.nb - wk.n), rows = 2 * nbg;
     const long long row0 = 2LL * ((long long)wk.pair * tb.nb + wk.n);
     const float wt = DENS ? __ldg(wk_ + wk.k) : 0.f;
-    const int2 pl = __ldg(tb.pl + wk.k);
+    const int2 pl = wk.pl;
     if (DENS && up && wk.pair >= tb.nk) {
       other_side();
       up = false;
@@ -339,9 +351,9 @@ __global__ void __launch_bounds__(Slab<N>::ITH, 2)
 #pragma unroll
       for (int j = 0; j < N; ++j) c[j * P] = a[j];
     }
-    __syncthreads();
     float2 *xp = xs + (vrow + row0) * rstride + (long long)z * tb.nnp;
     const float2 *u = us + row0 * rstride + (long long)z * tb.nnp;
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       const unsigned e = min(ft + i * TH, NN - 1);
