@@ -370,6 +370,7 @@ double fp64_clocks(double warps, double instr) {
 // 36 x 36 x 96 slab at 4 k points, updates included).  The FP32 fallback takes the same shapes.
 struct TnShape {
   int rm = 1, rn = 1, ty = 1, tx = 1, ntm = 1, ntn = 1, nsplit = 1;
+  double clocks = 0.0;
 };
 constexpr int kTnTiles[][2] = {{1, 1}, {2, 2}, {3, 3}, {4, 4}, {5, 5}, {4, 5}, {5, 4}};
 TnShape tn_shape(int M, int N, long long K, int batch) {
@@ -395,6 +396,7 @@ TnShape tn_shape(int M, int N, long long K, int batch) {
       if (tbest < 0.0 || t < tbest) {
         tbest = t;
         best = c;
+        best.clocks = t;
       }
     }
   }
@@ -493,6 +495,7 @@ __global__ void __launch_bounds__(128)
 // chunks where there are few columns.
 struct NnShape {
   int nr = 16, threads = 128;
+  double clocks = 0.0;
 };
 constexpr int kNnRows[] = {16, 14, 12, 10, 8, 4};
 NnShape nn_shape(int rows, long long ncol, int K, int batch) {
@@ -505,6 +508,7 @@ NnShape nn_shape(int rows, long long ncol, int K, int batch) {
     const double t = fp64_clocks(warps, nr * (4.0 * K + 2.0)) * (1.0 + 0.3 / nr);
     if (tbest < 0.0 || t < tbest) {
       tbest = t;
+      best.clocks = t;
       best.nr = nr;
       best.threads = warps >= 8 * 608 ? 128 : 32;
     }
@@ -539,11 +543,28 @@ __global__ void dmix_kernel(const cx<T> *__restrict__ proj, const cx<T> *__restr
   }
 }
 
+// tc: the FP64 form may run on the tensor cores (tc_gemm64_tn) where that is the faster
 template <class T>
 void gemm_tn(Context &ctx, DevBuf &partbuf, const cx<T> *A, long long lda, long long sA, int amod,
              const cx<T> *B, long long ldb, long long sB, cx<T> *C, long long sC, long long ldcm,
-             long long ldcn, int M, int N, long long K, int batch) {
+             long long ldcn, int M, int N, long long K, int batch, bool tc) {
   const TnShape c = tn_shape(M, N, K, batch);
+  auto reduce = [&](const cx<T> *part, int ns) {
+    const long long tot = (long long)batch * M * N;
+    const int th = spread_threads(tot, 1);
+    split_reduce_kernel<T><<<blocks_for(tot, th), th, 0, ctx.stream>>>(part, C, M, N, batch, ns,
+                                                                       sC, ldcm, ldcn);
+    TDLZ_LAUNCH_CHECK();
+  };
+  if constexpr (sizeof(T) == 8) {
+    double2 *part = nullptr;
+    int ns = 0;
+    if (tc && tc_gemm64_tn(ctx, partbuf, A, lda, sA, amod, B, ldb, sB, M, N, K, batch, c.clocks,
+                           part, ns)) {
+      reduce(part, ns);
+      return;
+    }
+  }
   const int nsplit = c.nsplit;
   size_t need = (size_t)nsplit * batch * M * N * sizeof(cx<T>);
   TDLZ_REQUIRE(need <= partbuf.bytes, TDLZ_ERR_STATE, "split-K scratch too small");
@@ -565,18 +586,15 @@ void gemm_tn(Context &ctx, DevBuf &partbuf, const cx<T> *A, long long lda, long 
     default: launch(gemm_tn_kernel<T, 5, 5>); break;
   }
   TDLZ_LAUNCH_CHECK();
-  long long tot = (long long)batch * M * N;
-  const int th = spread_threads(tot, 1);
-  split_reduce_kernel<T><<<blocks_for(tot, th), th, 0, ctx.stream>>>(
-      partbuf.template as<cx<T>>(), C, M, N, batch, nsplit, sC, ldcm, ldcn);
-  TDLZ_LAUNCH_CHECK();
+  reduce(pp, nsplit);
 }
 
+// tc, scratch: as in gemm_tn (tc_gemm64_nn)
 template <class T>
 void gemm_nn(Context &ctx, const cx<T> *A, long long sA, long long sar, long long sak,
              const cx<T> *B, long long ldb, long long sB, int bmod, const cx<T> *In, cx<T> *Out,
              long long ldo, long long sO, int rows, long long ncol, int K, T alpha, int batch,
-             int neg_from, int neg_mod = 1 << 30) {
+             int neg_from, int neg_mod, bool tc, DevBuf &scratch) {
   TDLZ_REQUIRE(K <= NN_KMAX, TDLZ_ERR_ARG, "contraction length above 256 (nocc or nproj)");
   auto launch = [&](auto kernel, int nc, int nr, int threads) {
     const dim3 grid((rows + nr - 1) / nr, (unsigned)((ncol + threads * nc - 1) / (threads * nc)),
@@ -592,6 +610,9 @@ void gemm_nn(Context &ctx, const cx<T> *A, long long sA, long long sar, long lon
     launch(gemm_nn_kernel<T, 2, 16>, 2, 16, 128);
   } else {
     const NnShape c = nn_shape(rows, ncol, K, batch);
+    if (tc && tc_gemm64_nn(ctx, scratch, A, sA, sar, sak, B, ldb, sB, bmod, In, Out, ldo, sO, rows,
+                           ncol, K, alpha, batch, neg_from, neg_mod, c.clocks))
+      return;
     switch (c.nr) {
       case 4: launch(gemm_nn_kernel<T, 1, 4>, 1, 4, c.threads); break;
       case 8: launch(gemm_nn_kernel<T, 1, 8>, 1, 8, c.threads); break;
@@ -1084,7 +1105,7 @@ void load_slot(Context &ctx, QSlot &s, const tdlz_ground_state *gs) {
     for (const DevBuf *u : {&d.ukq, &s.coeff_k}) {
       gemm_tn<double>(ctx, gpart, u->as<double2>(), 2LL * npwx, bstride, batch,
                       u->as<double2>(), 2LL * npwx, bstride, gram.as<double2>(),
-                      (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch);
+                      (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch, false);
       TDLZ_CUDA_TRY(cudaMemcpyAsync(g.data(), gram.p, g.size() * sizeof(double),
                                     cudaMemcpyDeviceToHost, st));
       TDLZ_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1433,7 +1454,7 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
     if (!tc)
       gemm_tn<T>(ctx, w.part, d.beta.template as<cx<T>>(), npwx, (long long)np_ * npwx, nk, x,
                  npwx, bstride, proj, (long long)np_ * 2 * nb, 2 * nb, 1, np_, 2 * nb, npwx,
-                 batch);
+                 batch, s.tensor_gemm);
     long long tot = (long long)batch * nb * 2 * np_;
     dmix_kernel<T><<<blocks_for(tot), kThreads, 0, st>>>(
         proj, d.dnl_val.template as<cx<T>>(), s.dnl_col.as<int>(), s.dnl_w, dm, np_, nb, batch);
@@ -1452,7 +1473,7 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
     if (!tcu)
       gemm_nn<T>(ctx, dm, (long long)2 * nb * np_, np_, 1, d.beta.template as<cx<T>>(), npwx,
                  (long long)np_ * npwx, nk, h, h, npwx, bstride, 2 * nb, npwx, np_, T(1), batch,
-                 batch);
+                 batch, 1 << 30, s.tensor_gemm, w.part);
   }
   // 8. P_c and the row sign (occupied k+q states shared: batch b -> (side, k) = b % 2nk;
   //    Y-side batches (b % 2nk >= nk) negated)
@@ -1468,7 +1489,7 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
                         ov, (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch);
     if (!tc)
       gemm_tn<T>(ctx, w.part, ukq, 2LL * npwx, bstride, batch1, h, 2LL * npwx, bstride, ov,
-                 (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch);
+                 (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch, s.tensor_gemm);
     bool tcu = false;
     if constexpr (sizeof(T) == 4)
       if (s.tensor_gemm) {
@@ -1482,7 +1503,8 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
       }
     if (!tcu)
       gemm_nn<T>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch1, h, y,
-                 2LL * npwx, bstride, nb, 2LL * npwx, nb, T(-1), batch, nk, batch1);
+                 2LL * npwx, bstride, nb, 2LL * npwx, nb, T(-1), batch, nk, batch1, s.tensor_gemm,
+                 w.part);
   }
   if (adj_mask) {
     ProfScope ps(pf, st, ST_LANCZOS, 2 * V * c, 0);
@@ -1509,13 +1531,15 @@ void start_vector(Context &ctx, QSlot &s, int mu, cx<T> *v) {
   double2 *ov = ovb.as<double2>();
   const double2 *ukq = s.d64.ukq.as<double2>();
   gemm_tn<double>(ctx, partb, ukq, 2LL * npwx, bstride, batch, tmp, 2LL * npwx, bstride, ov,
-                  (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch);
+                  (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch, s.tensor_gemm);
   if constexpr (sizeof(T) == 8) {
     gemm_nn<double>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch, tmp, v,
-                    2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch);
+                    2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch, 1 << 30,
+                    s.tensor_gemm, partb);
   } else {
     gemm_nn<double>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch, tmp, tmp,
-                    2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch);
+                    2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch, 1 << 30,
+                    s.tensor_gemm, partb);
     long long n = s.br_elems() * 2;
     convert_kernel<double, float><<<blocks_for(n), kThreads, 0, st>>>(
         reinterpret_cast<const double *>(tmp), reinterpret_cast<float *>(v), n);

@@ -1141,6 +1141,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                  "r"(g.tmem_cols));
 }
 
+#include "tc_gemm64.cuh"
+
 // ---------------------------------------------------------------------------------
 // Host side of the tensor-copy GEMMs.
 
@@ -1402,6 +1404,129 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
     tc_gemm_nn_img_kernel<<<(unsigned)nblocks, kTcThreads, smem, ctx.stream>>>(map, g);
     TDLZ_LAUNCH_CHECK();
   }
+  return true;
+}
+
+namespace {
+
+// Clocks of `tiles` tiles of nst stages over the persistent CTAs (one per SM): 72 MMAs or the
+// operands' split per stage, a drain every four and at the end, the outputs.  Taken below 0.7
+// of the FP64-pipe form's clocks: at 24 x 24 x 48, 18 bands, 4 k points (V_NL 0.101 ms by the pipe,
+// 0.100 by slices, P_c 0.114 and 0.105) the two meet.
+double oz_clocks(double tiles, double nst, int nt) {
+  const double tile = nst * 4500.0 + std::ceil(nst / kOzDrain) * 60.0 * nt + 4000.0;
+  return std::ceil(tiles / 152.0) * tile + 15000.0;
+}
+
+void oz_tiles(OzArgs &g) {
+  g.ntn = (g.M + kOzMaxNt / 2 - 1) / (kOzMaxNt / 2);
+  g.mt = (g.M + g.ntn - 1) / g.ntn;
+  g.nt = (2 * g.mt + 15) / 16 * 16;
+}
+
+template <bool NN> void oz_launch(Context &ctx, const OzArgs &g) {
+  // two stages and the raw elements; at least 116 KB: one CTA per SM (it takes all of TMEM)
+  const size_t smem = 2ull * kOzS * (kOzATile + (size_t)g.nt * kOzKT * 2) +
+                      16ull * 4 * (kOzSplit + 2 * kOzMaxNt);
+  const size_t ask = std::max(smem, (size_t)116 * 1024);
+  TDLZ_CUDA_TRY(cudaFuncSetAttribute(oz_gemm_kernel<NN>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ask));
+  oz_gemm_kernel<NN><<<(unsigned)std::min(152LL, g.tiles), kOzThreads, ask, ctx.stream>>>(g);
+  TDLZ_LAUNCH_CHECK();
+}
+
+}  // namespace
+
+bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda, long long sA,
+                  int amod, const double2 *B, long long ldb, long long sB, int M, int N,
+                  long long K, int batch, double clocks, double2 *&part, int &nsplit) {
+  if (batch % amod != 0 || K < 64) return false;
+  OzArgs g{};
+  g.A = A;
+  g.lda = lda;
+  g.sA = sA;
+  g.amod = amod;
+  g.B = B;
+  g.ldb = ldb;
+  g.sB = sB;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.batch = batch;
+  g.nj = batch / amod;
+  g.ntot = g.nj * N;
+  g.ntm = (g.ntot + 127) / 128;
+  oz_tiles(g);
+  const long long nst = (K + kOzKT / 2 - 1) / (kOzKT / 2);
+  const long long tiles = (long long)g.ntm * g.ntn * amod;
+  const size_t nexp = ((size_t)amod * M + (size_t)batch * N) * sizeof(int);
+  const size_t off = (nexp + 255) & ~(size_t)255, one = (size_t)batch * M * N * sizeof(double2);
+  if (partbuf.bytes < off + one) return false;
+  // K splits: whole drains, at most one wave of CTAs, within the scratch
+  long long ns = std::max(1LL, std::min(152 / tiles, (nst + 3) / 4));
+  ns = std::min(ns, (long long)((partbuf.bytes - off) / one));
+  const long long kst = ((nst + ns - 1) / ns + kOzDrain - 1) / kOzDrain * kOzDrain;
+  g.kst = (int)kst;
+  g.nsplit = (int)((nst + kst - 1) / kst);
+  g.tiles = tiles * g.nsplit;
+  if (kst > 1 << 16) return false;  // 2^14 drains: the sums stay below 2^63
+  if (oz_clocks((double)tiles * g.nsplit, (double)kst, g.nt) > 0.7 * clocks) return false;
+  int *e = partbuf.as<int>();
+  g.ea = e;
+  g.eb = e + (size_t)amod * M;
+  part = reinterpret_cast<double2 *>(partbuf.as<char>() + off);
+  g.part = part;
+  nsplit = g.nsplit;
+  const long long ra = (long long)amod * M, rb = (long long)batch * N;
+  oz_row_exp_kernel<<<(unsigned)ra, 128, 0, ctx.stream>>>(A, M, sA, lda, 1, K, e);
+  TDLZ_LAUNCH_CHECK();
+  oz_row_exp_kernel<<<(unsigned)rb, 128, 0, ctx.stream>>>(B, N, sB, ldb, 1, K, e + ra);
+  TDLZ_LAUNCH_CHECK();
+  oz_launch<false>(ctx, g);
+  return true;
+}
+
+bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA, long long sar,
+                  long long sak, const double2 *B, long long ldb, long long sB, int bmod,
+                  const double2 *In, double2 *Out, long long ldo, long long sO, int rows,
+                  long long ncol, int K, double alpha, int batch, int neg_from, int neg_mod,
+                  double clocks) {
+  OzArgs g{};
+  g.A = A;
+  g.sA = sA;
+  g.sar = sar;
+  g.sak = sak;
+  g.B = B;
+  g.ldb = ldb;
+  g.sB = sB;
+  g.amod = bmod;
+  g.M = rows;
+  g.K = K;
+  g.ncol = ncol;
+  g.batch = batch;
+  g.In = In;
+  g.Out = Out;
+  g.ldo = ldo;
+  g.sO = sO;
+  g.alpha = alpha;
+  g.neg_from = neg_from;
+  g.neg_mod = neg_mod;
+  oz_tiles(g);
+  g.nsplit = 1;
+  g.kst = (K + kOzKT / 2 - 1) / (kOzKT / 2);
+  g.ntm = (int)((ncol + 127) / 128);
+  g.tiles = (long long)g.ntm * g.ntn * batch;
+  if (oz_clocks((double)g.tiles, (double)g.kst, g.nt) > 0.7 * clocks) return false;
+  const long long ra = (long long)batch * rows, cb = (long long)bmod * ncol;
+  if (scratch.bytes < (size_t)(ra + cb) * sizeof(int)) return false;
+  int *e = scratch.as<int>();
+  g.ea = e;
+  g.eb = e + ra;
+  oz_row_exp_kernel<<<(unsigned)ra, 128, 0, ctx.stream>>>(A, rows, sA, sar, sak, K, e);
+  TDLZ_LAUNCH_CHECK();
+  oz_col_exp_kernel<<<blocks_for(cb), 256, 0, ctx.stream>>>(B, ldb, sB, bmod, K, ncol, e + ra);
+  TDLZ_LAUNCH_CHECK();
+  oz_launch<true>(ctx, g);
   return true;
 }
 

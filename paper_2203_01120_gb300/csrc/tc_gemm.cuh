@@ -41,6 +41,21 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
                     long long ldo, long long sO, int rows, float alpha, int batch, int neg_from,
                     int neg_mod);
 
+// FP64 contractions by exact integer slices on the tensor cores (tc_gemm64.cuh), where their
+// estimated clocks are below 0.7 of `clocks`, the estimate of the FP64-pipe form; otherwise
+// false, launching nothing.  The reduction writes its partial sums
+// part[z][b][m][n], z < nsplit, behind the row exponents in partbuf; the update needs
+// (batch rows + bmod ncol) ints of scratch.  Same contracts as tc_gemm_tn and tc_gemm_nn; a
+// row with a non-finite element gives NaN.
+bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda, long long sA,
+                  int amod, const double2 *B, long long ldb, long long sB, int M, int N,
+                  long long K, int batch, double clocks, double2 *&part, int &nsplit);
+bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA, long long sar,
+                  long long sak, const double2 *B, long long ldb, long long sB, int bmod,
+                  const double2 *In, double2 *Out, long long ldo, long long sO, int rows,
+                  long long ncol, int K, double alpha, int batch, int neg_from, int neg_mod,
+                  double clocks);
+
 // Throws TDLZ_ERR_TIMEOUT (and clears the flag) if a tensor-core GEMM gave up on an
 // mbarrier wait since the last check.  Synchronous.
 void tc_gemm_check();

@@ -1,0 +1,489 @@
+// FP64 contractions on the tensor cores by exact integer slices (included by tc_gemm.cu).
+//
+// The FP64 pipe of this part does 1.7 fused multiply-adds per clock and SM, the tensor cores
+// about 3600 in FP16.  Every operand row (along the contraction) is written as fixed-point
+// numbers of 62 bits below its largest exponent, and those as eight signed digits base 256:
+// x = 2^(e - 1084) sum_i d_i 256^(7 - i), -128 <= d_i <= 127, exact in FP16.  A product of
+// two digits has at most 2^14, so an FP32 accumulator holds the sum of the up to eight digit
+// pairs (i, j) with i + j = D over 128 terms exactly (8 x 128 x 2^14 = 2^24).  Eight
+// accumulators, D = 0..7 (36 of the 64 pairs; the rest lie 2^-62 below the rows' largest
+// products), sit side by side in TMEM; every 128 terms they are drained into two 64-bit
+// integers per output, and only the last step is FP64.  Nothing is rounded in between:
+// the error is the 62-bit quantisation of the rows, below the rounding of an FP64 sum unless
+// a row's largest element lies more than a factor of 2^9 above its typical one (the error-free
+// splitting of T. Ozaki, K. Ogita, S. Oishi, S. Rump, Numer. Algorithms 59,
+// 2012; on integer-valued tensor-core sums: Mukunoki et al., ISC 2020).
+//
+// One CTA per SM, with all 512 TMEM columns, walks its share of the (output tile of 128 rows x
+// nt <= 48 columns, K split) list, 32 reals of K per stage, two stages: sixteen warps copy the
+// next stage's operands (cp.async), split them (integer shifts and byte permutes, no FP64
+// instruction) and drain the accumulators, one more issues the 72 MMAs of a stage (issued by
+// one of the splitting warps they held up the others: 12000 clocks a stage).  Tiles follow
+// each other without a refill of the stages: with one CTA per tile the update's three stages
+// paid start and drain each time (V_NL and P_c of 0.52 and 0.67 ms for 0.38 and 0.41 below).
+// Bound by the split's integer instructions beside the 72 MMAs.  Measured, FP64 pipe -> slices,
+// one vector: 36 x 36 x 96 grid, 40 bands, 4 k points: V_NL 3.17 -> 0.55 ms, P_c 2.16 -> 0.59;
+// 45 x 45 x 144, 24 bands, 2 k points: V_NL 2.25 -> 0.38, P_c 0.93 -> 0.41.  Relative error of L x against
+// 64-bit sums: 1.298e-16 -> 1.278e-16 and 4.104e-16 -> 4.101e-16.
+#pragma once
+
+constexpr int kOzS = 8;                       // digits
+constexpr int kOzKT = 32;                     // reals of K per stage
+constexpr int kOzDrain = 4;                   // stages per drain (128 terms)
+constexpr uint32_t kOzATile = 128 * kOzKT * 2;  // bytes of one digit of the row operand
+constexpr int kOzMaxNt = 48;
+constexpr unsigned long long kOzBias = 0x8080808080808080ull;
+
+// biased exponent (at least 1) of |v|
+__device__ __forceinline__ int oz_exp(double v) {
+  return max(1, (__double2hiint(v) >> 20) & 0x7ff);
+}
+
+// digits of v below the row exponent e, as the bytes of fixed point + kOzBias (byte 7 first)
+__device__ __forceinline__ unsigned long long oz_fix(double v, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xfffffffffffffull;
+  if (ex) m |= 1ull << 52;
+  const int s = 9 - (e - max(ex, 1));
+  const unsigned long long q = s >= 0 ? m << s : s > -64 ? m >> -s : 0ull;
+  return ((long long)b < 0 ? 0ull - q : q) + kOzBias;
+}
+
+// FP16 pair (digit of x, digit of y) from byte `byte` of their fixed-point words
+__device__ __forceinline__ uint32_t oz_pair(unsigned long long x, unsigned long long y, int byte) {
+  const uint32_t xw = byte >= 4 ? (uint32_t)(x >> 32) : (uint32_t)x;
+  const uint32_t yw = byte >= 4 ? (uint32_t)(y >> 32) : (uint32_t)y;
+  const int s = byte & 3;
+  const uint32_t p =  // 1024 + byte of x, 1024 + byte of y
+      (__byte_perm(xw, yw, s | ((4 + s) << 8)) & 0x00ff00ffu) | 0x64006400u;
+  uint32_t r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(p), "r"(0x64806480u));  // - 1152
+  return r;
+}
+
+struct OzArgs {
+  const double2 *A, *B;  // TN: A[a][m][k], B[b][n][k]; NN: A[b][r][k] (strided), B[g][k][n]
+  long long lda, sA, ldb, sB, sar, sak;
+  int amod, M, N, nj, ntot, ntm, ntn, mt, nt, nsplit, batch, kst;  // kst: stages per split
+  long long K, ncol, tiles;
+  const int *ea, *eb;  // row exponents of A and of B (NN: of B's columns)
+  double2 *part;
+  const double2 *In;
+  double2 *Out;
+  long long ldo, sO;
+  double alpha;
+  int neg_from, neg_mod;
+};
+
+// max biased exponent of rows of len complex elements: row r starts at
+// p + (r / per) s0 + (r % per) s1, elements sk apart; one block per row
+__global__ void __launch_bounds__(128)
+    oz_row_exp_kernel(const double2 *__restrict__ p, int per, long long s0, long long s1,
+                      long long sk, long long len, int *__restrict__ e) {
+  const long long r = blockIdx.x;
+  const double2 *q = p + (r / per) * s0 + (r % per) * s1;
+  int m = 1;
+#pragma unroll 4
+  for (long long k = threadIdx.x; k < len; k += blockDim.x) {
+    const double2 v = q[k * sk];
+    m = max(m, max(oz_exp(v.x), oz_exp(v.y)));
+  }
+  __shared__ int sh[4];
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, sh[w]);
+    e[r] = m;
+  }
+}
+
+// max biased exponent of the columns n of B[g][k][n], k < K
+__global__ void oz_col_exp_kernel(const double2 *__restrict__ B, long long ldb, long long sB,
+                                  int G, int K, long long ncol, int *__restrict__ e) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= G * ncol) return;
+  const long long g = i / ncol;
+  const double2 *q = B + g * sB + (i - g * ncol);
+  int m = 1;
+  for (int k = 0; k < K; ++k) {
+    const double2 v = q[(long long)k * ldb];
+    m = max(m, max(oz_exp(v.x), oz_exp(v.y)));
+  }
+  e[i] = m;
+}
+
+// (hi 2^32 + lo) 2^e as a double, rounded once, without an FP64 instruction
+__device__ __forceinline__ double oz_value(long long hi, long long lo, int e) {
+  long long h = hi + (lo >> 32);
+  unsigned int l = (unsigned int)lo;  // value = h 2^32 + l
+  const bool neg = h < 0;
+  if (neg) {
+    h = l ? ~h : -h;
+    l = 0u - l;
+  }
+  if (h == 0 && l == 0) return 0.0;
+  const int z = h ? __clzll(h) : 64 + __clz(l);
+  unsigned long long m;  // the leading 64 bits
+  if (z == 0)
+    m = (unsigned long long)h;
+  else if (z < 64)
+    m = ((unsigned long long)h << z) | (z <= 32 ? (unsigned long long)l >> (32 - z)
+                                                : (unsigned long long)l << (z - 32));
+  else
+    m = (unsigned long long)l << (z - 32);
+  int x = 95 - z + e;  // exponent of the leading bit
+  m = (m >> 11) + ((m >> 10) & 1u);  // 53 bits, rounded half up
+  if (m >> 53) {
+    m >>= 1;
+    ++x;
+  }
+  if (x < -1022 || x > 1023) {
+    const double v = scalbn((double)m, x - 52);
+    return neg ? -v : v;
+  }
+  const unsigned long long b = ((unsigned long long)(x + 1023) << 52) | (m & 0xfffffffffffffull) |
+                               (neg ? 1ull << 63 : 0ull);
+  return __longlong_as_double((long long)b);
+}
+
+constexpr int kOzSplit = 512;                // threads of the splitting warps
+constexpr int kOzThreads = kOzSplit + 32;   // and the MMA warp
+
+// asynchronous 16-byte copy of a thread's own operand element into shared memory (zeros
+// where `in` is false)
+__device__ __forceinline__ void oz_copy(uint32_t dst, const double2 *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(in ? 16 : 0)
+               : "memory");
+}
+
+template <bool NN>
+__global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) {
+  extern __shared__ __align__(1024) unsigned char tc_smem[];
+  __shared__ __align__(8) uint64_t full[2], empty[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int bad;  // a wait expired
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nt = g.nt;
+  const uint32_t bTile = (uint32_t)nt * kOzKT * 2, lboA = 2048, lboB = (uint32_t)nt * 16;
+  const uint32_t stage_bytes = kOzS * (kOzATile + bTile);
+  // tiles [t0, t1) of this CTA, tile = ((z ntn + tn) ntm + tm): TN row tile tm of stacked
+  // (j, n), column tile tn of m, z = split amod + A batch; NN row tile of columns n, column
+  // tile of r, z = batch
+  const long long t0 = g.tiles * blockIdx.x / gridDim.x;
+  const long long t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
+  struct Tile {
+    int tm, tn, a, sp, b, bg, nst;
+    long long kc0;
+  };
+  auto tile_at = [&](long long t) {
+    Tile q;
+    q.tm = (int)(t % g.ntm);
+    t /= g.ntm;
+    q.tn = (int)(t % g.ntn);
+    const int z = (int)(t / g.ntn);
+    q.a = NN ? 0 : z % g.amod;
+    q.sp = NN ? 0 : z / g.amod;
+    q.b = NN ? z : 0;
+    q.bg = NN ? z % g.amod : 0;  // NN: amod holds bmod
+    q.kc0 = (long long)q.sp * g.kst * (kOzKT / 2);  // first complex k
+    q.nst = (int)min((long long)g.kst, (g.K - q.kc0 + kOzKT / 2 - 1) / (kOzKT / 2));
+    return q;
+  };
+  if (tid == 0) {
+    for (int s = 0; s < 2; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
+                   "r"(kOzSplit));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    bad = 0;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = tmem_slot;
+  if (warp == kOzSplit / 32) {
+    // ---- MMAs: stage u (counted over the CTA's tiles) holds its K tile once its 512 writers
+    // arrived (after the drain of the previous accumulators, where one was due)
+    if (lane == 0) {
+      const uint32_t idesc = (1u << 4)                        // D: F32; A, B: F16
+                             | ((uint32_t)(nt >> 3) << 17)    // N >> 3
+                             | ((uint32_t)(128 >> 4) << 24);  // M >> 4
+      int u = 0;
+      bool live = true;
+      for (long long t = t0; t < t1 && live; ++t) {
+        const int nst = tile_at(t).nst;
+        for (int it = 0; it < nst; ++it, ++u) {
+          const int s = u & 1;
+          if (!mbar_wait(smem_u32(&full[s]), (uint32_t)((u >> 1) & 1))) {
+            bad = 1;  // results are dropped; go on unless the stage really never came
+            if (!mbar_wait_raw(smem_u32(&full[s]), (uint32_t)((u >> 1) & 1))) {
+              live = false;
+              break;
+            }
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t ab = smem_u32(tc_smem + (size_t)s * stage_bytes);
+          const uint64_t da0 = smem_desc(ab, lboA, 128);
+          const uint64_t db0 = smem_desc(ab + kOzS * kOzATile, lboB, 128);
+          const uint32_t ea = kOzATile >> 4, eb = bTile >> 4;  // one digit on, in descriptors
+          for (int ks = 0; ks < kOzKT / 16; ++ks) {
+            const uint64_t dak = da0 + (uint64_t)(ks * (2 * lboA >> 4));
+            const uint64_t dbk = db0 + (uint64_t)(ks * (2 * lboB >> 4));
+            const bool fresh = (it & (kOzDrain - 1)) == 0 && ks == 0;
+#pragma unroll
+            for (int D = 0; D < kOzS; ++D)
+#pragma unroll
+              for (int i = 0; i <= D; ++i)
+                asm volatile(
+                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                        tmem + (uint32_t)(D * nt)),
+                    "l"(dak + (uint64_t)(i * ea)), "l"(dbk + (uint64_t)((D - i) * eb)),
+                    "r"(idesc), "r"((uint32_t)!(fresh && i == 0)));
+          }
+          asm volatile(
+              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                  smem_u32(&empty[s])));
+        }
+      }
+      // the last commit covers every MMA issued: wait for it before TMEM is released
+      if (u > 0) mbar_wait_raw(smem_u32(&empty[(u - 1) & 1]), (uint32_t)(((u - 1) >> 1) & 1));
+    }
+    __syncwarp();
+  } else {
+    // ---- one row unit per thread: row tid >> 2, chunk tid & 3 (TN: 4 lanes of a row read 256
+    // contiguous bytes) or row tid & 127, chunk tid >> 7 (NN: lanes read neighbouring
+    // columns); one column unit (pair row tid >> 2) for the tile's first threads
+    const int rrow = NN ? (tid & 127) : (tid >> 2), rch = NN ? (tid >> 7) : (tid & 3);
+    const int cm = tid >> 2, cc = tid & 3;
+    const double2 *rp = nullptr, *cp = nullptr;
+    int re = 1, ce = 1;
+    long long kc = 0;
+    int nst = 0;
+    auto operands = [&](long long t) {
+      const Tile q = tile_at(t);
+      kc = q.kc0;
+      nst = q.nst;
+      rp = cp = nullptr;
+      re = ce = 1;
+      const long long R = (long long)q.tm * 128 + rrow;
+      if (NN) {
+        if (R < g.ncol) {
+          rp = g.B + q.bg * g.sB + R;
+          re = g.eb[q.bg * g.ncol + R];
+        }
+      } else if (R < g.ntot) {
+        const int j = (int)(R / g.N), n = (int)(R - (long long)j * g.N);
+        const long long b = q.a + (long long)j * g.amod;
+        rp = g.B + b * g.sB + (long long)n * g.ldb;
+        re = g.eb[b * g.N + n];
+      }
+      const int cg = q.tn * g.mt + cm;
+      if (cm < g.mt && cg < g.M) {
+        cp = NN ? g.A + q.b * g.sA + (long long)cg * g.sar
+                : g.A + q.a * g.sA + (long long)cg * g.lda;
+        ce = NN ? g.ea[(long long)q.b * g.M + cg] : g.ea[(long long)q.a * g.M + cg];
+      }
+    };
+    // the thread's elements of a stage, copied a stage ahead: raw[u][thread], then the column
+    // units' (threads below 4 kOzMaxNt / 2)
+    constexpr int kCol = 2 * kOzMaxNt;
+    const uint32_t raw = smem_u32(tc_smem) + 2 * stage_bytes;
+    const uint32_t rrw = raw + 16u * tid, crw = raw + 16u * (4 * kOzSplit + tid);
+    auto copy = [&](int it) {
+      const long long k0 = kc + (long long)it * (kOzKT / 2);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const long long k = k0 + 4 * rch + u;
+        const bool in = rp && k < g.K;
+        oz_copy(rrw + 16u * kOzSplit * u, in ? (NN ? rp + k * g.ldb : rp + k) : g.B, in);
+      }
+      if (tid < kCol) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const long long k = k0 + 4 * cc + u;
+          const bool in = cp && k < g.K;
+          oz_copy(crw + 16u * kCol * u, in ? (NN ? cp + k * g.sak : cp + k) : g.A, in);
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto fetch = [](uint32_t at) {
+      double2 v;
+      asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(at) : "memory");
+      return v;
+    };
+    // warp w drains lanes 32 (w & 3) .., columns (w >> 2) nt / 4 ..: nt / 4 = 4, 8 or 12
+    long long hi[kOzMaxNt / 4], lo[kOzMaxNt / 4];
+#pragma unroll
+    for (int i = 0; i < kOzMaxNt / 4; ++i) hi[i] = lo[i] = 0;
+    const int quarter = warp & 3, cq = warp >> 2, ngrp = nt >> 4;
+    // the accumulators into hi (D = 0..3) and lo (D = 4..7); all MMAs on them are done
+    auto drain = [&] {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+      for (int q = 0; q < kOzMaxNt / 16; ++q) {
+        if (q < ngrp) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t r[4][4];
+#pragma unroll
+            for (int D = 0; D < 4; ++D) {
+              const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) +
+                                     (uint32_t)((4 * h + D) * nt + cq * (nt >> 2) + 4 * q);
+              asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                           : "=r"(r[D][0]), "=r"(r[D][1]), "=r"(r[D][2]), "=r"(r[D][3])
+                           : "r"(taddr));
+            }
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              int f[4];
+#pragma unroll
+              for (int D = 0; D < 4; ++D) f[D] = __float2int_rn(__uint_as_float(r[D][u]));
+              long long &t = h ? lo[4 * q + u] : hi[4 * q + u];
+              t += ((long long)f[0] * 256 + f[1]) * 65536 + ((long long)f[2] * 256 + f[3]);
+            }
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+    };
+    // an expired wait drops the results (ok); after one that really never came, none is waited
+    // for again
+    bool ok = true, dead = false;
+    auto arrived = [&](int s, int phase) {
+      const uint32_t at = smem_u32(&empty[s]);
+      bool in = !dead && mbar_wait(at, (uint32_t)(phase & 1));
+      if (!in && !dead) dead = !mbar_wait_raw(at, (uint32_t)(phase & 1));
+      ok = __all_sync(0xffffffffu, in) && ok;  // uniform: the drain's loads want whole warps
+    };
+    // outputs of a tile: row 32 quarter + lane; columns (2m, 2m + 1) = (Re, Im); sums cleared
+    auto output = [&](long long t) {
+      const Tile q = tile_at(t);
+      const long long R = (long long)q.tm * 128 + 32 * quarter + lane;
+      if (R < (NN ? g.ncol : (long long)g.ntot)) {
+        const int j = NN ? 0 : (int)(R / g.N), n = NN ? 0 : (int)(R - (long long)j * g.N);
+        const long long b = NN ? q.b : q.a + (long long)j * g.amod;
+        const int er = NN ? g.eb[q.bg * g.ncol + R] : g.eb[b * g.N + n];
+        const int m0 = q.tn * g.mt + cq * (nt >> 3);
+        const int nm = min(min(nt >> 3, g.mt - cq * (nt >> 3)), g.M - m0);
+        const int *ep = g.ea + (NN ? b : (long long)q.a) * g.M + m0;
+        const long long at = NN ? b * g.sO + (long long)m0 * g.ldo + R
+                                : (((long long)q.sp * g.batch + b) * g.M + m0) * g.N + n;
+        const double sg = NN && (q.b % g.neg_mod) >= g.neg_from ? -1.0 : 1.0;
+#pragma unroll
+        for (int c = 0; c < kOzMaxNt / 8; ++c)
+          if (c < nm) {
+            const int em = ep[c];
+            double2 v;
+            v.x = oz_value(hi[2 * c], lo[2 * c], er + em - 2112);
+            v.y = oz_value(hi[2 * c + 1], lo[2 * c + 1], er + em - 2112);
+            if (er == 0x7ff || em == 0x7ff || !ok)  // non-finite operand, or expired wait
+              v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+            if (NN) {
+              const double2 iv = g.In[at + (long long)c * g.ldo];
+              g.Out[at + (long long)c * g.ldo] =
+                  make_double2(sg * fma(g.alpha, v.x, iv.x), sg * fma(g.alpha, v.y, iv.y));
+            } else {
+              g.part[at + (long long)c * g.N] = v;
+            }
+          }
+      }
+#pragma unroll
+      for (int i = 0; i < kOzMaxNt / 4; ++i) hi[i] = lo[i] = 0;
+    };
+    int u = 0;
+    if (t0 < t1) {
+      operands(t0);
+      copy(0);
+    }
+    for (long long t = t0; t < t1; ++t) {
+      const int n = nst;
+      for (int it = 0; it < n; ++it, ++u) {
+        const int s = u & 1;
+        if (u >= 2) arrived(s, (u - 2) >> 1);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        unsigned char *st = tc_smem + (size_t)s * stage_bytes;
+        unsigned long long x[4], y[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const double2 v = fetch(rrw + 16u * kOzSplit * w);
+          x[w] = oz_fix(v.x, re);
+          y[w] = oz_fix(v.y, re);
+        }
+        unsigned char *o = st + tile_off(rrow, rch, lboA);
+#pragma unroll
+        for (int d = 0; d < kOzS; ++d)
+          *reinterpret_cast<uint4 *>(o + d * kOzATile) =
+              make_uint4(oz_pair(x[0], y[0], 7 - d), oz_pair(x[1], y[1], 7 - d),
+                         oz_pair(x[2], y[2], 7 - d), oz_pair(x[3], y[3], 7 - d));
+        if (2 * cm < nt) {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            const double2 v = fetch(crw + 16u * kCol * w);
+            x[w] = oz_fix(v.x, ce);
+            y[w] = oz_fix(v.y, ce);
+          }
+          unsigned char *oc = st + kOzS * kOzATile;
+#pragma unroll
+          for (int d = 0; d < kOzS; ++d) {
+            uint32_t p[4], q[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              // TN: Re row (x, y), Im row (-y, x); NN: Re row (x, -y), Im row (y, x)
+              const uint32_t h = oz_pair(x[w], y[w], 7 - d), sw = __byte_perm(h, 0, 0x1032);
+              p[w] = NN ? h ^ 0x80000000u : h;
+              q[w] = NN ? sw : sw ^ 0x00008000u;
+            }
+            *reinterpret_cast<uint4 *>(oc + d * bTile + tile_off(2 * cm, cc, lboB)) =
+                make_uint4(p[0], p[1], p[2], p[3]);
+            *reinterpret_cast<uint4 *>(oc + d * bTile + tile_off(2 * cm + 1, cc, lboB)) =
+                make_uint4(q[0], q[1], q[2], q[3]);
+          }
+        }
+        // this thread's elements of the next stage (its own slots: no barrier needed)
+        if (it + 1 < n) {
+          copy(it + 1);
+        } else if (t + 1 < t1) {
+          operands(t + 1);
+          copy(0);
+        }
+        const bool due = u > 0 && (it & (kOzDrain - 1)) == 0;
+        if (due) {
+          // the next MMAs start the accumulators afresh: drain them first
+          arrived(s ^ 1, (u - 1) >> 1);
+          drain();
+        }
+        // an expired wait still arrives, so that the MMA warp and the other writers run on
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[s]))
+                     : "memory");
+        if (due && it == 0) output(t - 1);  // under the MMAs of the new tile
+      }
+    }
+    if (u > 0) {
+      arrived((u - 1) & 1, (u - 1) >> 1);
+      if (!ok) bad = 1;
+      asm volatile("bar.sync 1, %0;" ::"n"(kOzSplit) : "memory");
+      ok = __all_sync(0xffffffffu, ok && !bad);
+      drain();
+      output(t1 - 1);
+      if (!ok && lane == 0) atomicExch(&g_tc_timeout, 1);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
