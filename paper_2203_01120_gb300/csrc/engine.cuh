@@ -141,6 +141,10 @@ struct QSlot {
   bool slab_planes = false;
   DevBuf slab_pl;   // [nk] int2 (planes from j1 = 0 up, planes in all)
   DevBuf slab_pos;  // [nk][nstick_max]
+  // FP64 lines on the tensor cores (lines64.cuh), axes X and Y: largest |m1|, |m2| of the
+  // spheres, matrix images
+  int ln_h[2] = {0, 0};
+  DevBuf ln_img[2];
   bool slab32 = false;  // the FP32 Liouvillian's steps 1-6 run the slab stages
   int dnl_w = 0;   // nonzeros per row of D in the ELL form (padded)
   DevBuf dnl_col;  // [2nproj][dnl_w] column of each entry of dnl_val, -1 past the row's end

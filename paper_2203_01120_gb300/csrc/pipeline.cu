@@ -20,6 +20,7 @@
 
 #include "pipeline.cuh"
 #include "regfft.cuh"
+#include "tc_gemm.cuh"
 
 // Launch KERNEL<T, N>(args) for the register-line lengths; sets ok = false otherwise.
 // (rt: threads per CTA, a variable in the calling scope)
@@ -1003,6 +1004,31 @@ void build_stick_tables(QSlot &s, const std::vector<int> &idx_kq) {
   up(s.st_id, sid);
   s.nst_h = nst;
   s.npl_h = npl;
+  // largest |m1|, |m2| (grid index j stands for j or j - n), the line matrices
+  s.ln_h[0] = s.ln_h[1] = 0;
+  for (int k = 0; k < nk; ++k)
+    for (int c : sticks[k]) {
+      const int j1 = c / n2, j2 = c % n2;
+      s.ln_h[0] = std::max(s.ln_h[0], std::min(j1, n1 - j1));
+      s.ln_h[1] = std::max(s.ln_h[1], std::min(j2, n2 - j2));
+    }
+  for (int a = 0; a < 2; ++a) {
+    std::vector<uint16_t> img;
+    if (!tc_lines_build(s.fft[a], s.ln_h[a], img)) continue;
+    s.ln_img[a].alloc(img.size() * sizeof(uint16_t));
+    TDLZ_CUDA_TRY(cudaMemcpy(s.ln_img[a].p, img.data(), s.ln_img[a].bytes, cudaMemcpyHostToDevice));
+  }
+}
+
+// FP64 lines on the tensor cores, where they run
+template <class T> bool takes_slices(const QSlot &s, int axis) {
+  return sizeof(T) == 8 && tc_lines_taken(s, axis);
+}
+template <class T>
+bool slice_lines(Context &ctx, QSlot &s, int axis, bool inverse, const cx<T> *src, cx<T> *dst,
+                 long long rows) {
+  if constexpr (sizeof(T) == 8) return tc_lines(ctx, s, axis, inverse, src, dst, rows);
+  return false;
 }
 
 // Element counts and FLOPs of one pass over nvec stacked vectors, for the
@@ -1096,8 +1122,8 @@ void pipeline_inverse(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *xr, cx<T> *
   // sticks in, planes out and back in, real-space grids out
   ProfScope ps(ctx.prof, st, ST_FFT_INV, wk.S1 * c + 2 * wk.S2 * c + wk.G * c,
                wk.y_flops + wk.x_flops);
-  ok = use_reg_lines<T>(n2);
-  if (ok) {
+  ok = slice_lines<T>(ctx, s, 1, true, i1, i2, rows);
+  if (!ok && (ok = use_reg_lines<T>(n2))) {
     tuned_lines(ctx, "inv_y", c, n2, (long long)npm * n3, rows, [&](int rt) {
       dim3 g = grid_rows((unsigned)(((long long)npm * n3 + rt - 1) / rt), rows);
       TDLZ_REG_LAUNCH(n2, inv_y_reg_kernel, g, i1, i2, s.pl_n.as<int>(), s.st_id.as<int>(),
@@ -1113,8 +1139,8 @@ void pipeline_inverse(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *xr, cx<T> *
         stages(s.plan.ax[1]), tw_of<T>(s.plan.ax[1]));
     TDLZ_LAUNCH_CHECK();
   }
-  ok = use_reg_lines<T>(n1);
-  if (ok) {
+  ok = slice_lines<T>(ctx, s, 0, true, i2, xr, rows);
+  if (!ok && (ok = use_reg_lines<T>(n1))) {
     tuned_lines(ctx, "inv_x", c, n1, n23, rows, [&](int rt) {
       dim3 g = grid_rows((unsigned)((n23 + rt - 1) / rt), rows);
       TDLZ_REG_LAUNCH(n1, inv_x_reg_kernel, g, i2, xr, s.pl_of.as<int>(), s.nk, s.nb, npm, n23,
@@ -1144,7 +1170,7 @@ void pipeline_forward(Context &ctx, QSlot &s, const cx<T> *x, const cx<T> *xr, c
   const StageWork wk = stage_work<T>(s, nvec);
   // potentials of every vector and the local fields, read once per point
   const double pot_bytes = 4.0 * nvec * s.nr * (c + sizeof(T));
-  bool ok = use_reg_lines<T>(n1);
+  bool ok = use_reg_lines<T>(n1) || takes_slices<T>(s, 0);
   if (ok) {
     // products in place (xr is not needed afterwards): x(r) read and written, U(r)
     // once per stacked group
@@ -1166,14 +1192,15 @@ void pipeline_forward(Context &ctx, QSlot &s, const cx<T> *x, const cx<T> *xr, c
     }
     ProfScope ps(ctx.prof, st, ST_FFT_FWD, wk.G * c + 2 * wk.S2 * c + wk.S1 * c,
                  wk.x_flops + wk.y_flops);
-    tuned_lines(ctx, "fwd_x", c, n1, n23, rows, [&](int rt) {
-      dim3 g = grid_rows((unsigned)((n23 + rt - 1) / rt), rows);
-      TDLZ_REG_LAUNCH(n1, fwd_x_reg_kernel, g, xr, i2, s.pl_of.as<int>(), s.nk, s.nb, npm, n23,
-                      s.nr, rows);
-      TDLZ_LAUNCH_CHECK();
-    });
-    ok = use_reg_lines<T>(n2);
-    if (ok) {
+    if (!slice_lines<T>(ctx, s, 0, false, xr, i2, rows))
+      tuned_lines(ctx, "fwd_x", c, n1, n23, rows, [&](int rt) {
+        dim3 g = grid_rows((unsigned)((n23 + rt - 1) / rt), rows);
+        TDLZ_REG_LAUNCH(n1, fwd_x_reg_kernel, g, xr, i2, s.pl_of.as<int>(), s.nk, s.nb, npm, n23,
+                        s.nr, rows);
+        TDLZ_LAUNCH_CHECK();
+      });
+    ok = slice_lines<T>(ctx, s, 1, false, i2, i1, rows);
+    if (!ok && (ok = use_reg_lines<T>(n2))) {
       tuned_lines(ctx, "fwd_y", c, n2, (long long)npm * n3, rows, [&](int rt) {
         dim3 gy = grid_rows((unsigned)(((long long)npm * n3 + rt - 1) / rt), rows);
         TDLZ_REG_LAUNCH(n2, fwd_y_reg_kernel, gy, i2, i1, s.pl_n.as<int>(), s.st_id.as<int>(),
@@ -1201,8 +1228,8 @@ void pipeline_forward(Context &ctx, QSlot &s, const cx<T> *x, const cx<T> *xr, c
                                          s.pl_j1.as<int>(), s.nk, s.nb, npm, n1, n23, s.nr, nbs,
                                          stages(s.plan.ax[0]), tw_of<T>(s.plan.ax[0]));
     TDLZ_LAUNCH_CHECK();
-    ok = use_reg_lines<T>(n2);
-    if (ok) {
+    ok = slice_lines<T>(ctx, s, 1, false, i2, i1, rows);
+    if (!ok && (ok = use_reg_lines<T>(n2))) {
       tuned_lines(ctx, "fwd_y", c, n2, (long long)npm * n3, rows, [&](int rt) {
         dim3 gy = grid_rows((unsigned)(((long long)npm * n3 + rt - 1) / rt), rows);
         TDLZ_REG_LAUNCH(n2, fwd_y_reg_kernel, gy, i2, i1, s.pl_n.as<int>(), s.st_id.as<int>(),

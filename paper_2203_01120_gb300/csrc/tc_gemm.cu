@@ -1142,6 +1142,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 }
 
 #include "tc_gemm64.cuh"
+#include "lines64.cuh"
 
 // ---------------------------------------------------------------------------------
 // Host side of the tensor-copy GEMMs.
@@ -1527,6 +1528,137 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
   oz_col_exp_kernel<<<blocks_for(cb), 256, 0, ctx.stream>>>(B, ldb, sB, bmod, K, ncol, e + ra);
   TDLZ_LAUNCH_CHECK();
   oz_launch<true>(ctx, g);
+  return true;
+}
+
+namespace {
+
+// cos and sin of 2 pi t / n, scaled by 2^58 and rounded: Taylor sums in 62-bit fixed point over
+// the first octant (integers only: the same on every host)
+void fixed_cos_sin(long long t, long long n, long long &c, long long &s) {
+  long long num = 2 * (t % n), den = n;  // angle = pi num / den
+  bool neg_s = false, neg_c = false;
+  if (num > den) {
+    num = 2 * den - num;
+    neg_s = true;
+  }
+  if (2 * num > den) {
+    num = den - num;
+    neg_c = true;
+  }
+  const bool swap = 4 * num > den;
+  if (swap) {
+    num = den - 2 * num;
+    den *= 2;
+  }
+  const __int128 pi = (__int128)0xC90FDAA22168C235ull;  // pi 2^62
+  const __int128 x = (pi * num + den / 2) / den, x2 = (x * x) >> 62;
+  __int128 tc = (__int128)1 << 62, ts = x, sc = tc, ss = ts;
+  for (int i = 1; i < 14; ++i) {
+    tc = -((tc * x2) >> 62) / ((2 * i - 1) * (2 * i));
+    ts = -((ts * x2) >> 62) / ((2 * i) * (2 * i + 1));
+    sc += tc;
+    ss += ts;
+  }
+  c = (long long)((sc + 8) >> 4);
+  s = (long long)((ss + 8) >> 4);
+  if (swap) std::swap(c, s);
+  if (neg_c) c = -c;
+  if (neg_s) s = -s;
+}
+
+uint16_t half_bits(int d) {  // |d| < 2048
+  if (d == 0) return 0;
+  const int a = std::abs(d), e = 31 - __builtin_clz((unsigned)a);
+  return (uint16_t)((d < 0 ? 0x8000 : 0) | (e + 15) << 10 | ((a << (10 - e)) & 0x3ff));
+}
+
+}  // namespace
+
+bool tc_lines_build(int n, int h, std::vector<uint16_t> &img) {
+  if (n > 48 || h > 15 || 2 * h >= n) return false;
+  img.assign(kLnB, 0);  // both directions: kLnB bytes each
+  for (int dir = 0; dir < 2; ++dir) {
+    const int cols = dir ? 16 : 32, nhalf = dir ? 2 : 1;
+    const int nmax = dir ? n / 2 : h, kmax = dir ? h : n / 2;
+    for (int cs = 0; cs < 2; ++cs)
+      for (int k = 0; k <= kmax; ++k) {
+        const int row = (k & 3) * (cols / 4) + (k >> 2);
+        double bound[kLnD] = {};  // of the accumulators
+        for (int hh = 0; hh < nhalf; ++hh)
+          for (int kk = 0; kk < 16; ++kk) {
+            const int m = 16 * hh + (kk >> 2) + 4 * (kk & 3);  // index n of term kk
+            if (m > nmax) continue;
+            long long c, s;
+            fixed_cos_sin((long long)m * k, n, c, s);
+            const unsigned long long w = (unsigned long long)(cs ? s : c) + kLnBias;
+            int dg[kLnD];
+            for (int j = 0; j < kLnD; ++j) {
+              dg[j] = (int)((w >> (10 * (kLnD - 1 - j))) & 1023) - 512;
+              const int br = j * cols + row;  // the digits' columns side by side
+              const size_t byte = dir * (size_t)kLnB + (size_t)(cs * nhalf + hh) * kLnD * cols * 32 +
+                                  (size_t)(kk >> 3) * kLnD * cols * 16 + (br >> 3) * 128 +
+                                  (br & 7) * 16 + (kk & 7) * 2;
+              img[byte / 2] = half_bits(dg[j]);
+            }
+            for (int D = 0; D < kLnD; ++D)
+              for (int i = 0; i <= D; ++i) bound[D] += (i ? 512.0 : 257.0) * std::abs(dg[D - i]);
+          }
+        for (double b : bound)
+          if (b > 16777216.0) return false;
+      }
+  }
+  return true;
+}
+
+template <bool INV, bool Y> void tc_lines_launch(Context &ctx, const LineArgs &g) {
+  // the A stages, the matrix and the raw elements: one CTA per SM (it takes all of TMEM)
+  const size_t smem = 4 * kLnD * kLnA + kLnB + 8 * (INV ? 8 : 16) * kOzSplit;
+  TDLZ_CUDA_TRY(cudaFuncSetAttribute(line_kernel<INV, Y>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  line_kernel<INV, Y><<<(unsigned)std::min(152LL, g.tiles), kOzThreads, smem, ctx.stream>>>(g);
+  TDLZ_LAUNCH_CHECK();
+}
+
+bool tc_lines_taken(const QSlot &s, int axis) {
+  const long long nl = (axis ? s.nplane_max : (long long)s.fft[1]) * s.fft[2];
+  return s.tensor_gemm && s.ln_img[axis].p && s.nr < 1 << 27 && (nl + 63) / 64 * s.rows() >= kLnMinTiles;
+}
+
+bool tc_lines(Context &ctx, QSlot &s, int axis, bool inverse, const double2 *src, double2 *dst,
+              long long rows) {
+  if (!tc_lines_taken(s, axis)) return false;
+  LineArgs g{};
+  const long long n2 = s.fft[1], n3 = s.fft[2];
+  g.src = src;
+  g.dst = dst;
+  g.img = s.ln_img[axis].as<char>() + (inverse ? 0 : kLnB);
+  g.N = s.fft[axis];
+  g.h = s.ln_h[axis];
+  g.nk = s.nk;
+  g.nb = s.nb;
+  g.npm = s.nplane_max;
+  g.n3 = (int)n3;
+  if (axis == 0) {
+    g.tab = s.pl_of.as<int>();
+    g.nl = (int)(n2 * n3);
+    g.st = (int)(n2 * n3 * sizeof(double2));
+    g.sp = g.npm * n2 * n3;
+    g.sf = s.nr;
+  } else {
+    g.tab = s.st_id.as<int>();
+    g.npl = s.pl_n.as<int>();
+    g.nl = (int)(g.npm * n3);
+    g.st = (int)(n3 * sizeof(double2));
+    g.sp = s.nstick_max * n3;
+    g.sf = g.npm * n2 * n3;
+  }
+  g.tpr = (g.nl + 63) / 64;
+  g.tiles = (long long)g.tpr * rows;
+  if (axis == 0)
+    inverse ? tc_lines_launch<true, false>(ctx, g) : tc_lines_launch<false, false>(ctx, g);
+  else
+    inverse ? tc_lines_launch<true, true>(ctx, g) : tc_lines_launch<false, true>(ctx, g);
   return true;
 }
 

@@ -56,6 +56,18 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
                   long long ncol, int K, double alpha, int batch, int neg_from, int neg_mod,
                   double clocks);
 
+// X (axis 0) or Y (axis 1) line transforms of the FP64 pipeline on the tensor cores
+// (lines64.cuh), between its packed and full buffers (inverse: packed to full).  Returns false,
+// launching nothing, where the axis has no matrix image or there are few lines; the caller
+// then uses the register or Stockham lines.
+bool tc_lines(Context &ctx, QSlot &s, int axis, bool inverse, const double2 *src, double2 *dst,
+              long long rows);
+bool tc_lines_taken(const QSlot &s, int axis);
+
+// Both directions' matrix images of length n with packed entries at |index| <= h; false for
+// n > 48, h > 15, 2 h >= n, or sums beyond the accumulators' exact range.
+bool tc_lines_build(int n, int h, std::vector<uint16_t> &img);
+
 // Throws TDLZ_ERR_TIMEOUT (and clears the flag) if a tensor-core GEMM gave up on an
 // mbarrier wait since the last check.  Synchronous.
 void tc_gemm_check();

@@ -60,3 +60,49 @@ def test_slices(cell, nocc, natom, nk, monkeypatch):
     for key in ("alpha", "beta", "gamma"):
         a, b = np.asarray(run["0"][key]), np.asarray(run["1"][key])
         assert np.allclose(a, b, rtol=1e-11, atol=1e-11 * np.abs(a).max()), key
+
+
+@pytest.mark.parametrize("fft,ecut,nk,nocc", [
+    ((15, 18, 20), 3.6, 4, 24), ((24, 25, 27), 12.0, 2, 20), ((32, 30, 36), 20.0, 2, 10),
+    ((40, 45, 24), 12.0, 2, 20), ((48, 32, 32), 20.0, 1, 22), ((54, 48, 20), 12.0, 2, 30)])
+def test_slice_lines(fft, ecut, nk, nocc, monkeypatch):
+    """X and Y lines by slices: even and odd lengths up to 48, one and two halves of the
+    forward sum, lengths without a register transform, ragged last tiles, and 54 (another line
+    transform).  Same bars; scaled by 1e-290 (results near
+    the end of the normal range) and zero."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import synth.configs as sc
+    from oracle.liouvillian import Liouvillian
+    from paper_2203_01120_gb300 import TDLZ_FP64, Context, build
+    from synth import random_br_vector
+    build()
+    monkeypatch.setitem(sc.CONFIGS, "_lines64", dataclasses.replace(
+        sc.CONFIGS["C0"], name="C0", fft=fft, ecut=ecut, nocc=nocc, kgrid=(1, nk, 1), seed=41))
+    gs = sc.make_ground_state("_lines64", solver="random")
+    x = random_br_vector(gs, seed=8)
+    ref = Liouvillian(gs).apply(x)
+    y = {}
+    for tc in "01":
+        monkeypatch.setenv("TDLZ_TC", tc)
+        ctx = Context(0)
+        try:
+            q = ctx.load_ground_state(gs)
+            for scale in (1.0, 1e-290, 0.0):
+                xt = torch.as_tensor(x * scale, device="cuda")
+                yt = torch.empty_like(xt)
+                torch.cuda.synchronize()
+                ctx.apply_liouvillian(q, xt, yt, False, TDLZ_FP64)
+                ctx.synchronize()
+                got = yt.cpu().numpy()
+                if scale == 0.0:
+                    assert not got.any()
+                    continue
+                err = np.linalg.norm(got / scale - ref) / np.linalg.norm(ref)
+                assert err <= 1e-12, (tc, scale, err)
+                y.setdefault(tc, got)
+        finally:
+            ctx.close()
+    assert not np.array_equal(y["0"], y["1"])
+    assert np.linalg.norm(y["1"] - y["0"]) <= 1e-13 * np.linalg.norm(ref)
