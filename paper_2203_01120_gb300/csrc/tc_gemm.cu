@@ -1410,7 +1410,7 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
 
 namespace {
 
-// Clocks of `tiles` tiles of nst stages over the persistent CTAs (one per SM): 72 MMAs or the
+// Clocks of `tiles` tiles of nst stages over the persistent CTAs (one per SM): the MMAs or the
 // operands' split per stage, a drain every four and at the end, the outputs.  Taken below 0.7
 // of the FP64-pipe form's clocks: at 24 x 24 x 48, 18 bands, 4 k points (V_NL 0.101 ms by the pipe,
 // 0.100 by slices, P_c 0.114 and 0.105) the two meet.

@@ -17,14 +17,16 @@
 // One CTA per SM, with all 512 TMEM columns, walks its share of the (output tile of 128 rows x
 // nt <= 48 columns, K split) list, 32 reals of K per stage, two stages: sixteen warps copy the
 // next stage's operands (cp.async), split them (integer shifts and byte permutes, no FP64
-// instruction) and drain the accumulators, one more issues the 72 MMAs of a stage (issued by
-// one of the splitting warps they held up the others: 12000 clocks a stage).  Tiles follow
+// instruction) and drain the accumulators, one more issues the MMAs of a stage (issued by
+// one of the splitting warps they held up the others: 12000 clocks a stage).  A row digit is
+// multiplied by its 8 - i column digits side by side in one or two MMAs, so that it is read
+// twice at most (one MMA per pair: 7% more time).  Tiles follow
 // each other without a refill of the stages: with one CTA per tile the update's three stages
 // paid start and drain each time (V_NL and P_c of 0.52 and 0.67 ms for 0.38 and 0.41 below).
-// Bound by the split's integer instructions beside the 72 MMAs.  Measured, FP64 pipe -> slices,
-// one vector: 36 x 36 x 96 grid, 40 bands, 4 k points: V_NL 3.17 -> 0.55 ms, P_c 2.16 -> 0.59;
-// 45 x 45 x 144, 24 bands, 2 k points: V_NL 2.25 -> 0.38, P_c 0.93 -> 0.41.  Relative error of L x against
-// 64-bit sums: 1.298e-16 -> 1.278e-16 and 4.104e-16 -> 4.101e-16.
+// Bound by the split's integer instructions beside the MMAs.  Measured, FP64 pipe -> slices,
+// one vector: 36 x 36 x 96 grid, 40 bands, 4 k points: V_NL 3.17 -> 0.51 ms, P_c 2.16 -> 0.57;
+// 45 x 45 x 144, 24 bands, 2 k points: V_NL 2.25 -> 0.36, P_c 0.93 -> 0.39.  Relative error of
+// L x against 64-bit sums: 1.298e-16 -> 1.278e-16 and 4.104e-16 -> 4.101e-16.
 #pragma once
 
 constexpr int kOzS = 8;                       // digits
@@ -167,7 +169,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
   __shared__ int bad;  // a wait expired
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nt = g.nt;
-  const uint32_t bTile = (uint32_t)nt * kOzKT * 2, lboA = 2048, lboB = (uint32_t)nt * 16;
+  const uint32_t bTile = (uint32_t)nt * kOzKT * 2, lboA = 2048;
+  const uint32_t lboB = (uint32_t)(kOzS * nt) * 16;  // the column digits' rows side by side
   const uint32_t stage_bytes = kOzS * (kOzATile + bTile);
   // tiles [t0, t1) of this CTA, tile = ((z ntn + tn) ntm + tm): TN row tile tm of stacked
   // (j, n), column tile tn of m, z = split amod + A batch; NN row tile of columns n, column
@@ -216,8 +219,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
     // arrived (after the drain of the previous accumulators, where one was due)
     if (lane == 0) {
       const uint32_t idesc = (1u << 4)                        // D: F32; A, B: F16
-                             | ((uint32_t)(nt >> 3) << 17)    // N >> 3
-                             | ((uint32_t)(128 >> 4) << 24);  // M >> 4
+                             | ((uint32_t)(128 >> 4) << 24);  // M >> 4; N >> 3 at bit 17
       int u = 0;
       bool live = true;
       for (long long t = t0; t < t1 && live; ++t) {
@@ -235,21 +237,25 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
           const uint32_t ab = smem_u32(tc_smem + (size_t)s * stage_bytes);
           const uint64_t da0 = smem_desc(ab, lboA, 128);
           const uint64_t db0 = smem_desc(ab + kOzS * kOzATile, lboB, 128);
-          const uint32_t ea = kOzATile >> 4, eb = bTile >> 4;  // one digit on, in descriptors
+          const uint32_t ea = kOzATile >> 4;  // one digit on, in descriptors
           for (int ks = 0; ks < kOzKT / 16; ++ks) {
             const uint64_t dak = da0 + (uint64_t)(ks * (2 * lboA >> 4));
             const uint64_t dbk = db0 + (uint64_t)(ks * (2 * lboB >> 4));
             const bool fresh = (it & (kOzDrain - 1)) == 0 && ks == 0;
+            // digit i of the rows by digits 0 .. 7 - i of the columns, side by side, in parts of
+            // at most 256 columns: accumulators i .. 7
 #pragma unroll
-            for (int D = 0; D < kOzS; ++D)
-#pragma unroll
-              for (int i = 0; i <= D; ++i)
+            for (int i = 0; i < kOzS; ++i) {
+              const int all = (kOzS - i) * nt, most = 256 / nt * nt;
+              for (int c0 = 0; c0 < all; c0 += most)
                 asm volatile(
                     "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                        tmem + (uint32_t)(D * nt)),
-                    "l"(dak + (uint64_t)(i * ea)), "l"(dbk + (uint64_t)((D - i) * eb)),
-                    "r"(idesc), "r"((uint32_t)!(fresh && i == 0)));
+                        tmem + (uint32_t)(i * nt + c0)),
+                    "l"(dak + (uint64_t)(i * ea)), "l"(dbk + (uint64_t)(c0 >> 3) * 8),
+                    "r"(idesc | (uint32_t)(min(most, all - c0) >> 3) << 17),
+                    "r"((uint32_t)!(fresh && i == 0)));
+            }
           }
           asm volatile(
               "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -446,9 +452,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
               p[w] = NN ? h ^ 0x80000000u : h;
               q[w] = NN ? sw : sw ^ 0x00008000u;
             }
-            *reinterpret_cast<uint4 *>(oc + d * bTile + tile_off(2 * cm, cc, lboB)) =
+            *reinterpret_cast<uint4 *>(oc + tile_off(d * nt + 2 * cm, cc, lboB)) =
                 make_uint4(p[0], p[1], p[2], p[3]);
-            *reinterpret_cast<uint4 *>(oc + d * bTile + tile_off(2 * cm + 1, cc, lboB)) =
+            *reinterpret_cast<uint4 *>(oc + tile_off(d * nt + 2 * cm + 1, cc, lboB)) =
                 make_uint4(q[0], q[1], q[2], q[3]);
           }
         }
