@@ -22,10 +22,25 @@
 #include "regfft.cuh"
 #include "tc_gemm.cuh"
 
-// Launch KERNEL<T, N>(args) for the register-line lengths; sets ok = false otherwise.
-// (rt: threads per CTA, a variable in the calling scope)
+// Launch KERNEL<T, N>(args) for the register-line lengths (line_length); sets ok = false
+// otherwise.  (rt: threads per CTA, a variable in the calling scope)
+#define TDLZ_REG_CASE(KERNEL, N, grid, ...)                                            \
+  case N:                                                                            \
+    if constexpr (sizeof(T) == 4)                                                    \
+      KERNEL<T, N><<<grid, rt, 0, st>>>(__VA_ARGS__, regtw<T, N>());                   \
+    else                                                                             \
+      ok = false;                                                                    \
+    break;
 #define TDLZ_REG_LAUNCH(n, KERNEL, grid, ...)                                          \
   switch (n) {                                                                       \
+    TDLZ_REG_CASE(KERNEL, 15, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 18, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 20, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 25, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 27, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 30, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 32, grid, __VA_ARGS__)                                       \
+    TDLZ_REG_CASE(KERNEL, 40, grid, __VA_ARGS__)                                       \
     case 12: KERNEL<T, 12><<<grid, rt, 0, st>>>(__VA_ARGS__, regtw<T, 12>()); break; \
     case 16: KERNEL<T, 16><<<grid, rt, 0, st>>>(__VA_ARGS__, regtw<T, 16>()); break; \
     case 24: KERNEL<T, 24><<<grid, rt, 0, st>>>(__VA_ARGS__, regtw<T, 24>()); break; \
@@ -875,9 +890,12 @@ inline void z_plan(int n3, int &n1, int &n2) {
     else ok = false;                                                                     \
   } while (0)
 
-// Register-line transforms: FP32 up to length 48, FP64 up to 45 (spill-free budget).
+// Register-line transforms: FP32 up to length 48, FP64 up to 45 (spill-free budget) without the
+// lengths between (its larger grids run slices, lines64.cuh).
 template <class T> bool use_reg_lines(int n) {
-  return reg_fft_length(n) && (sizeof(T) == 4 || n <= 45);
+  if (sizeof(T) == 8) return reg_fft_length(n) && n <= 45;
+  return reg_fft_length(n) || n == 15 || n == 18 || n == 20 || n == 25 || n == 27 || n == 30 ||
+         n == 32 || n == 40;
 }
 
 }  // namespace

@@ -31,6 +31,18 @@ def _ground_state(fft, nocc):
                                  (45, 45, 16), (36, 36, 48), (12, 12, 96), (12, 12, 144),
                                  (16, 16, 192), (36, 24, 12), (16, 48, 45)])
 def test_register_lines(fft):
+    _check(fft, 3)
+
+
+@pytest.mark.parametrize("fft", [(15, 18, 12), (18, 15, 20), (20, 25, 27), (25, 20, 16),
+                                 (27, 30, 40), (30, 27, 12), (32, 40, 24), (40, 32, 30)])
+@pytest.mark.parametrize("nocc", [1, 5])
+def test_register_lines_between(fft, nocc):
+    """The lengths between on both axes, with few bands (the reductions' K splits)."""
+    _check(fft, nocc)
+
+
+def _check(fft, nocc):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -38,7 +50,7 @@ def test_register_lines(fft):
     from paper_2203_01120_gb300 import TDLZ_FP64, TDLZ_MIXED, Context, build
     from synth import random_br_vector
     build()
-    gs = _ground_state(fft, 3)
+    gs = _ground_state(fft, nocc)
     x = random_br_vector(gs, seed=5)
     lv = Liouvillian(gs)
     flip = np.array([1.0, -1.0])[:, None, None, None, None]
