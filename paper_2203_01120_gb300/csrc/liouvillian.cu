@@ -815,7 +815,17 @@ void alloc_workspace(QSlot &s, int nvec) {
   w.ovl.alloc(batch * s.nb * s.nb * c);
   size_t p1 = (size_t)32 * batch * std::max(s.nproj, 1) * 2 * s.nb;
   size_t p2 = (size_t)32 * batch * s.nb * s.nb;
-  w.part.alloc(std::max(p1, p2) * c);
+  // at least 32 K splits of the tensor-core reductions (a few bands at one or two k points leave
+  // them as few CTAs; 30 x 25 x 40 grid, 11 bands, 2 k points: 5 and 8 splits fitted)
+  size_t p3 = 0;
+  if (sizeof(T) == 4 && s.tensor_gemm)
+    for (const auto &[groups, cols] : {std::pair<size_t, size_t>{s.nk, nv * 4 * s.nb},
+                                       std::pair<size_t, size_t>{2 * s.nk, nv * s.nb}}) {
+      const size_t tiles = (cols + 255) / 256;
+      p3 = std::max(p3, 32 * groups * tiles * 128 *
+                            (((cols + tiles - 1) / tiles + 15) / 16 * 16) * sizeof(float));
+    }
+  w.part.alloc(std::max(std::max(p1, p2) * c, p3));
   w.nvec_cap = nvec;
   w.ready = true;
 }

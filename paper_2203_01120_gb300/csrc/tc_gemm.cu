@@ -813,7 +813,8 @@ bool tc_gemm_tn_transposed(Context &ctx, DevBuf &partbuf, const float2 *A, long 
   tc_gemm_tnt_kernel<<<grid, kTcThreads, smem, ctx.stream>>>(g);
   TDLZ_LAUNCH_CHECK();
   const long long total = (long long)batch * M * N;
-  tc_reduce_t_kernel<<<blocks_for(total), 256, 0, ctx.stream>>>(g.part, C, M, N, amod, g.nj,
+  const int th = spread_threads(total, 1);
+  tc_reduce_t_kernel<<<blocks_for(total, th), th, 0, ctx.stream>>>(g.part, C, M, N, amod, g.nj,
                                                                  g.ntiles, g.nm, g.nsplit, sC,
                                                                  ldcm, ldcn);
   TDLZ_LAUNCH_CHECK();
@@ -1245,7 +1246,8 @@ bool tc_gemm_tn(Context &ctx, DevBuf &partbuf, const float2 *A, long long lda, l
   tc_gemm_tn_kernel<<<grid, kTcThreads, smem, ctx.stream>>>(g);
   TDLZ_LAUNCH_CHECK();
   const long long total = (long long)batch * M * N;
-  tc_reduce_kernel<<<blocks_for(total), 256, 0, ctx.stream>>>(g.part, C, M, N, amod, g.nj,
+  const int th = spread_threads(total, 1);
+  tc_reduce_kernel<<<blocks_for(total, th), th, 0, ctx.stream>>>(g.part, C, M, N, amod, g.nj,
                                                                g.ntiles, g.nt, g.nsplit, sC,
                                                                ldcm, ldcn);
   TDLZ_LAUNCH_CHECK();
