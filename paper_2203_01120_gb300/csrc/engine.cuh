@@ -199,7 +199,8 @@ template <class T> void ensure_precision(Context &ctx, QSlot &s);
 template <class T>
 void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nvec,
                        unsigned adj_mask);
-template <class T> void start_vector(Context &ctx, QSlot &s, int mu, cx<T> *v);
+template <class T>
+void start_vectors(Context &ctx, QSlot &s, const int *mu, int m, cx<T> *v, double2 *tmp);
 // y = L x (or L^H x) for one vector in the caller's plane-wave order (x, y device).
 template <class T>
 void apply_liouvillian_caller_order(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y,

@@ -579,7 +579,6 @@ void ChainSet::init_impl() {
     gr.nv = flavor == TDLZ_NONHERMITIAN ? 2 * m : m;
     const int nslot = flavor == TDLZ_PSEUDOHERMITIAN_POSDEF ? 4 : 3;
     gr.vec.alloc((size_t)nslot * gr.nv * n * c);
-    TDLZ_CUDA_TRY(cudaMemsetAsync(gr.vec.p, 0, gr.vec.bytes, ctx->stream));
     for (int k = 0; k < nslot; ++k) gr.slot[k] = (char *)gr.vec.p + (size_t)k * gr.nv * n * c;
     for (int mi = 0; mi < m; ++mi) {
       Chain &ch = chains[gr.members[mi]];
@@ -592,8 +591,13 @@ void ChainSet::init_impl() {
       ch.cf.beta = reinterpret_cast<double *>(ch.cf.z + 4 * (size_t)cap);
       ch.sc.alloc(sizeof(ChainScalars));
       TDLZ_CUDA_TRY(cudaMemsetAsync(ch.sc.p, 0, ch.sc.bytes, ctx->stream));
-      start_vector<T>(*ctx, s, ch.mu, (cx<T> *)gr.slot[0] + mi * n);
     }
+    std::vector<int> mu;
+    for (int i : gr.members) mu.push_back(chains[i].mu);
+    // the slots after the first (at least m FP64 vectors) are its scratch, zeroed afterwards
+    start_vectors<T>(*ctx, s, mu.data(), m, (cx<T> *)gr.slot[0], (double2 *)gr.slot[1]);
+    const size_t first = (size_t)gr.nv * n * c;
+    TDLZ_CUDA_TRY(cudaMemsetAsync(gr.slot[1], 0, gr.vec.bytes - first, ctx->stream));
     if (flavor == TDLZ_PSEUDOHERMITIAN_POSDEF)  // w = L v for every member, one pass
       apply_liouvillian<T>(*ctx, s, (cx<T> *)gr.slot[0], (cx<T> *)gr.slot[3], m, 0u);
     double2 *part = red.as<double2>();

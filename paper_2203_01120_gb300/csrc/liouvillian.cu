@@ -1523,37 +1523,51 @@ void apply_liouvillian(Context &ctx, QSlot &s, const cx<T> *x, cx<T> *y, int nve
   }
 }
 
-// v^mu = (P sigma^mu U, P+ sigma^mu T U) on the k+q spheres (Sec. 2.5).
+// v^mu = (P sigma^mu U, P+ sigma^mu T U) on the k+q spheres (Sec. 2.5) for m components, one
+// after the other in v; tmp holds m FP64 vectors.  Up to four share the overlap and update
+// launches: an overlap tile of 128 rows holds three components' 40 bands as one's.
+// Chain creation, FP32, 36 x 36 x 96 grid, 40 bands, 16 k points, three components: 9.0 ms one
+// component at a time with scratch of its own, 5.5 like this.
 template <class T>
-void start_vector(Context &ctx, QSlot &s, int mu, cx<T> *v) {
+void start_vectors(Context &ctx, QSlot &s, const int *mu, int m, cx<T> *v, double2 *tmp) {
   cudaStream_t st = ctx.stream;
   const int nk = s.nk, nb = s.nb, npwx = s.npwx;
-  const int batch = 2 * nk;
-  const long long bstride = (long long)nb * 2 * npwx;
-  DevBuf tmpb, ovb, partb;
-  tmpb.alloc((size_t)s.br_elems() * sizeof(double2));
-  ovb.alloc((size_t)batch * nb * nb * sizeof(double2));
-  partb.alloc((size_t)32 * batch * nb * nb * sizeof(double2));
-  double2 *tmp = tmpb.as<double2>();
-  sigma_u_kernel<double><<<blocks_for(2LL * nk * nb * npwx), kThreads, 0, st>>>(
-      s.coeff_k.as<double2>(), s.map_kq_k.as<int>(), mu, tmp, nk, nb, npwx, 1.0);
-  TDLZ_LAUNCH_CHECK();
+  const int batch1 = 2 * nk, most = std::min(m, 4);
+  const long long bstride = (long long)nb * 2 * npwx, br = s.br_elems();
+  DevBuf ovb, partb;
+  ovb.alloc((size_t)most * batch1 * nb * nb * sizeof(double2));
+  // K splits: the FP64-pipe form's, or a tile of the slices per SM; row exponents of the slices
+  const int last = m % most ? m % most : most;
+  const int splits = std::max({tn_shape(nb, nb, 2LL * npwx, most * batch1).nsplit,
+                               tn_shape(nb, nb, 2LL * npwx, last * batch1).nsplit,
+                               std::min(32, 1 + 152 / batch1)});
+  const size_t outs = (size_t)most * batch1 * nb * nb;
+  partb.alloc(splits * outs * sizeof(double2) +
+              ((size_t)(most + 1) * batch1 * (nb + 2LL * npwx) + 64) * sizeof(int));
   double2 *ov = ovb.as<double2>();
   const double2 *ukq = s.d64.ukq.as<double2>();
-  gemm_tn<double>(ctx, partb, ukq, 2LL * npwx, bstride, batch, tmp, 2LL * npwx, bstride, ov,
-                  (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch, s.tensor_gemm);
-  if constexpr (sizeof(T) == 8) {
-    gemm_nn<double>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch, tmp, v,
+  for (int c0 = 0; c0 < m; c0 += most) {
+    const int mc = std::min(most, m - c0), batch = mc * batch1;
+    cx<T> *vc = v + c0 * br;
+    for (int c = 0; c < mc; ++c) {
+      sigma_u_kernel<double><<<blocks_for(2LL * nk * nb * npwx), kThreads, 0, st>>>(
+          s.coeff_k.as<double2>(), s.map_kq_k.as<int>(), mu[c0 + c], tmp + c * br, nk, nb, npwx,
+          1.0);
+      TDLZ_LAUNCH_CHECK();
+    }
+    gemm_tn<double>(ctx, partb, ukq, 2LL * npwx, bstride, batch1, tmp, 2LL * npwx, bstride, ov,
+                    (long long)nb * nb, nb, 1, nb, nb, 2LL * npwx, batch, s.tensor_gemm);
+    double2 *out = tmp;
+    if constexpr (sizeof(T) == 8) out = vc;
+    gemm_nn<double>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch1, tmp, out,
                     2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch, 1 << 30,
                     s.tensor_gemm, partb);
-  } else {
-    gemm_nn<double>(ctx, ov, (long long)nb * nb, 1, nb, ukq, 2LL * npwx, bstride, batch, tmp, tmp,
-                    2LL * npwx, bstride, nb, 2LL * npwx, nb, -1.0, batch, batch, 1 << 30,
-                    s.tensor_gemm, partb);
-    long long n = s.br_elems() * 2;
-    convert_kernel<double, float><<<blocks_for(n), kThreads, 0, st>>>(
-        reinterpret_cast<const double *>(tmp), reinterpret_cast<float *>(v), n);
-    TDLZ_LAUNCH_CHECK();
+    if constexpr (sizeof(T) == 4) {
+      const long long n = mc * br * 2;
+      convert_kernel<double, float><<<blocks_for(n), kThreads, 0, st>>>(
+          reinterpret_cast<const double *>(tmp), reinterpret_cast<float *>(vc), n);
+      TDLZ_LAUNCH_CHECK();
+    }
   }
   TDLZ_CUDA_TRY(cudaStreamSynchronize(st));
 }
@@ -1596,8 +1610,8 @@ template void apply_liouvillian<double>(Context &, QSlot &, const double2 *, dou
                                         unsigned);
 template void apply_liouvillian<float>(Context &, QSlot &, const float2 *, float2 *, int,
                                        unsigned);
-template void start_vector<double>(Context &, QSlot &, int, double2 *);
-template void start_vector<float>(Context &, QSlot &, int, float2 *);
+template void start_vectors<double>(Context &, QSlot &, const int *, int, double2 *, double2 *);
+template void start_vectors<float>(Context &, QSlot &, const int *, int, float2 *, double2 *);
 template void apply_liouvillian_caller_order<double>(Context &, QSlot &, const double2 *,
                                                      double2 *, bool);
 template void apply_liouvillian_caller_order<float>(Context &, QSlot &, const float2 *,

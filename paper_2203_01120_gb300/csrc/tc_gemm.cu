@@ -1465,15 +1465,24 @@ bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda
   const size_t nexp = ((size_t)amod * M + (size_t)batch * N) * sizeof(int);
   const size_t off = (nexp + 255) & ~(size_t)255, one = (size_t)batch * M * N * sizeof(double2);
   if (partbuf.bytes < off + one) return false;
-  // K splits: whole drains, at most one wave of CTAs, within the scratch
-  long long ns = std::max(1LL, std::min(152 / tiles, (nst + 3) / 4));
-  ns = std::min(ns, (long long)((partbuf.bytes - off) / one));
-  const long long kst = ((nst + ns - 1) / ns + kOzDrain - 1) / kOzDrain * kOzDrain;
+  // K splits of whole drains, within the scratch: the number whose tiles the CTAs walk soonest
+  // (96 tiles of 1500 stages, one split: 1500 stage times; three: 1000)
+  long long kst = 0;
+  double best = 0.0;
+  const long long most = std::min({(nst + 3) / 4, (long long)((partbuf.bytes - off) / one), 64LL});
+  for (long long ns = 1; ns <= most; ++ns) {
+    const long long st = ((nst + ns - 1) / ns + kOzDrain - 1) / kOzDrain * kOzDrain;
+    const double t = oz_clocks((double)tiles * ((nst + st - 1) / st), (double)st, g.nt);
+    if (kst == 0 || t < best) {
+      best = t;
+      kst = st;
+    }
+  }
   g.kst = (int)kst;
   g.nsplit = (int)((nst + kst - 1) / kst);
   g.tiles = tiles * g.nsplit;
   if (kst > 1 << 16) return false;  // 2^14 drains: the sums stay below 2^63
-  if (oz_clocks((double)tiles * g.nsplit, (double)kst, g.nt) > 0.7 * clocks) return false;
+  if (best > 0.7 * clocks) return false;
   int *e = partbuf.as<int>();
   g.ea = e;
   g.eb = e + (size_t)amod * M;
@@ -1598,8 +1607,8 @@ bool tc_lines_build(int n, int h, std::vector<uint16_t> &img) {
             for (int j = 0; j < kLnD; ++j) {
               dg[j] = (int)((w >> (10 * (kLnD - 1 - j))) & 1023) - 512;
               const int br = j * cols + row;  // the digits' columns side by side
-              const size_t byte = dir * (size_t)kLnB + (size_t)(cs * nhalf + hh) * kLnD * cols * 32 +
-                                  (size_t)(kk >> 3) * kLnD * cols * 16 + (br >> 3) * 128 +
+              const size_t byte = dir * (size_t)kLnB +
+                                  (size_t)(cs * nhalf + hh) * kLnD * cols * 32 + (size_t)(kk >> 3) * kLnD * cols * 16 + (br >> 3) * 128 +
                                   (br & 7) * 16 + (kk & 7) * 2;
               img[byte / 2] = half_bits(dg[j]);
             }
@@ -1624,7 +1633,8 @@ template <bool INV, bool Y> void tc_lines_launch(Context &ctx, const LineArgs &g
 
 bool tc_lines_taken(const QSlot &s, int axis) {
   const long long nl = (axis ? s.nplane_max : (long long)s.fft[1]) * s.fft[2];
-  return s.tensor_gemm && s.ln_img[axis].p && s.nr < 1 << 27 && (nl + 63) / 64 * s.rows() >= kLnMinTiles;
+  return s.tensor_gemm && s.ln_img[axis].p && s.nr < 1 << 27 &&
+         (nl + 63) / 64 * s.rows() >= kLnMinTiles;
 }
 
 bool tc_lines(Context &ctx, QSlot &s, int axis, bool inverse, const double2 *src, double2 *dst,
