@@ -287,15 +287,14 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-# DRAM bytes per launch of a stage's kernel, from one ncu capture of the same build
-# (dram__bytes_read.sum + dram__bytes_write.sum): the product kernel of the C2 step
-# (6 stacked vectors) captured at 4 of the 16 k points, scaled by 4 (its traffic is
-# linear in the number of k points).  Summary: profiles/kernels_C2_k4_full.md.
-NCU_TRAFFIC = {("C2", "product"): 4 * 8.837e9}
+# DRAM bytes per launch of a stage's kernel (dram__bytes_read.sum + dram__bytes_write.sum), for
+# the stages that have been captured at the benchmark's size.
+NCU_TRAFFIC = {}
 
 
-# GB300's FP64 vector rate (nominal, dense): the binding roof of the FP64 path, whose
-# FFT, pointwise and GEMM stages all run on the FP64 pipe.
+# GB300's FP64 vector rate (nominal, dense), the roof of the FP64 path's pointwise stages and Z
+# lines; its X and Y lines and contractions run as integer slices on the tensor cores, so that
+# the path's nominal FP64 flops can exceed this rate.
 FP64_PEAK_TFLOPS = 1.25
 
 
@@ -640,8 +639,12 @@ def run_tdlz(args):
         nsm, npm = sphere_sticks_planes(gs)
         cufft["pruned"] = cufft_pruned_baseline(rows, fft, nsm, npm, local)
         st_ms = {k: v["ms"] / args.steps for k, v in prof.items()}
-        cufft["tdlz_inverse_ms"] = st_ms.get("scatter", 0.0) + st_ms.get("fft_inv", 0.0)
-        cufft["tdlz_forward_ms"] = st_ms.get("fft_fwd", 0.0) + st_ms.get("gather", 0.0)
+        inv, fwd = st_ms.get("fft_inv", 0.0), st_ms.get("fft_fwd", 0.0)
+        # slab stages: the Y and X lines run inside the density and the product stage
+        cufft["tdlz_inverse_ms"] = st_ms.get("scatter", 0.0) + (inv or st_ms.get("density", 0.0))
+        cufft["tdlz_forward_ms"] = st_ms.get("gather", 0.0) + (fwd or st_ms.get("product", 0.0))
+        cufft["tdlz_includes"] = ("lines only" if inv else
+                                  "inverse: the density sums; forward: the products")
     batched = run_batched(args, local, stream) if args.batched else None
     if rank != 0:
         return

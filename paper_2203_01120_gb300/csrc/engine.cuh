@@ -90,6 +90,7 @@ template <class T> struct SlotData {
 
 template <class T> struct Workspace {
   DevBuf xr;    // staged pipeline: [nvec][2][nk][nb][2][Nr] real-space response orbitals
+                // (slab stages: in z-plane order)
   DevBuf rho;   // [nvec][4][Nr]
   DevBuf rhopart;  // [groups][nvec][4][Nr] partial densities
   DevBuf vpot;  // [nvec][4][Nr]; plane stages: potential planes [nvec][n3][6][n1*n2 (even)]
@@ -99,9 +100,9 @@ template <class T> struct Workspace {
   DevBuf proj;  // [2nk][nproj][2nb]  <beta|x>
   DevBuf dmix;  // [2nk][2nb][nproj]
   DevBuf ovl;   // [2nk][nb][nb]      <U_kq|h>
-  DevBuf part;  // split-K partial sums
+  DevBuf part;  // split-K partial sums, row exponents of the FP64 slices
   DevBuf i1;    // stick scratch: [rows][nstick_max][n3]; plane stages [rows][n3][nstick_max]
-  DevBuf i2;    // staged pipeline: [rows][nplane_max][n2][n3] plane scratch
+  DevBuf i2;    // staged pipeline without slab stages: [rows][nplane_max][n2][n3] plane scratch
   int nvec_cap = 0;  // stacked vectors the buffers above are sized for
   int ns_cap = 1;    // staged pipeline: vectors per sub-batch its grids are sized for
   bool ready = false;

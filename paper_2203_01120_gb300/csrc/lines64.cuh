@@ -24,7 +24,9 @@
 // grid, 40 bands, 4 k points: 3.10 -> 1.47 and 3.09 -> 1.42 ms; 45 x 45 x 144, 24 bands, 2 k
 // points: 2.71 -> 0.92 and 2.70 -> 0.88; three vectors of 24 x 24 x 48, 18 bands, 4 k points:
 // 1.48 -> 1.09 and 1.47 -> 0.94.  Relative error of L x against 64-bit sums: 1.298e-16 ->
-// 1.285e-16, 4.104e-16 -> 4.101e-16, 3.119e-16 -> 3.120e-16.
+// 1.285e-16, 4.104e-16 -> 4.101e-16, 3.119e-16 -> 3.120e-16; of single lines of 12 to 48 points
+// against 80-bit sums (the integer steps on the host): 4.6e-17 to 5.7e-17, an FP64 FFT's 1.1e-16
+// to 2.1e-16.
 #pragma once
 
 constexpr int kLnD = 6;                        // digits

@@ -1059,7 +1059,7 @@ void load_slot(Context &ctx, QSlot &s, const tdlz_ground_state *gs) {
   s.plan.init(gs->fft);
   build_stick_tables(s, idx_kq);
   // Real-space stages, per precision: the staged pipeline (real-space grids of the stacked
-  // vectors in HBM, in sub-batches that take at most a tenth of the device) where one
+  // vectors in HBM, in sub-batches that fit the device) where one
   // vector's buffers take at most 30% of the device memory; otherwise the fused plane
   // stages, whose workspace is the stick buffer.  Where both fit, the staged pipeline is
   // the faster (its grid traffic costs less HBM time than the plane stages' extra line

@@ -8,12 +8,15 @@
 //   Y: only the planes that hold sticks, lines assembled from the stick buffer,
 //   X: every column, lines assembled from the plane buffer -> x(r),
 // and the forward transform mirrors it:
-//   X: every column, with [v_loc + s B.sigma] x + W^s U formed while loading
-//      (the product stage is fused), keeping only the sphere's planes,
+//   X: every column of [v_loc + s B.sigma] x + W^s U (formed by a pass before, or while
+//      loading where the length has no register transform), keeping only the sphere's planes,
 //   Y: keeping only the sphere's sticks,
 //   Z: writing only sphere coefficients, fused with + (|k+q+G|^2/2 - e_n) x.
-// Each pass runs the Stockham line transform of fft.cu's axis kernel on a tile
-// of TL lines held in shared memory as [position][TL + 1].
+// Lines run in one thread's registers where the length allows it (regfft.cuh), FP64 X and Y
+// lines of larger grids as integer slices on the tensor cores (lines64.cuh); otherwise a pass
+// runs the Stockham line transform of fft.cu's axis kernel on a tile of TL lines held in
+// shared memory as [position][TL + 1].  In FP32 on square grids the slab stages (slab.cu) take
+// the place of the X and Y passes and use the Z passes alone.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

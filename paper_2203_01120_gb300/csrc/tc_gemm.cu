@@ -1607,8 +1607,9 @@ bool tc_lines_build(int n, int h, std::vector<uint16_t> &img) {
             for (int j = 0; j < kLnD; ++j) {
               dg[j] = (int)((w >> (10 * (kLnD - 1 - j))) & 1023) - 512;
               const int br = j * cols + row;  // the digits' columns side by side
-              const size_t byte = dir * (size_t)kLnB +
-                                  (size_t)(cs * nhalf + hh) * kLnD * cols * 32 + (size_t)(kk >> 3) * kLnD * cols * 16 + (br >> 3) * 128 +
+              const size_t block = (size_t)(cs * nhalf + hh) * kLnD * cols * 32;
+              const size_t byte = dir * (size_t)kLnB + block +
+                                  (size_t)(kk >> 3) * kLnD * cols * 16 + (br >> 3) * 128 +
                                   (br & 7) * 16 + (kk & 7) * 2;
               img[byte / 2] = half_bits(dg[j]);
             }
