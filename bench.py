@@ -298,6 +298,11 @@ NCU_TRAFFIC = {}
 FP64_PEAK_TFLOPS = 1.25
 
 
+# stages whose arithmetic stays on the FP64 pipe on this workload (the X and Y lines and the
+# contractions run as integer slices on the tensor cores)
+FP64_PIPE_STAGES = ("scatter", "density", "hartree", "potential", "product", "gather", "lanczos")
+
+
 def fp64_roofline(prof64):
     """Nominal flops of the profiled FP64 steps (per stage: 5 N log2 N per line transform,
     8 per complex multiply-add of the contractions, the pointwise products) over their
@@ -691,7 +696,9 @@ def run_tdlz(args):
         "fp64": None if sps_fp64 is None else {
             "value": sps_fp64, "unit": "steps/s", "steps": fp64_steps,
             "ms_per_step": 1000 * wall_fp64 / fp64_steps,
-            "roofline": fp64_roofline(prof64)},
+            "roofline": fp64_roofline({k: v for k, v in prof64.items()
+                                       if k in FP64_PIPE_STAGES}),
+            "roofline_stages": list(FP64_PIPE_STAGES)},
         "chi": chi,
         "roofline": {
             "bound": "alu", "achieved": achieved_tf, "peak": peak32, "unit": "TFLOP/s",
