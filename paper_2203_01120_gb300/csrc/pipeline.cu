@@ -513,7 +513,8 @@ __global__ void __launch_bounds__(kZThreads)
       const int l0 = blockIdx.x * LPB + (threadIdx.x >> 5) * Z::LW;
       const int nv = min(max(__ldg(nst + k) - l0, 0), Z::LW);
       int4 *wd = zd[threadIdx.x >> 5];
-      if (lane <= nv) wd[lane] = __ldg(runs + (long long)k * (nsm + 1) + l0 + lane);
+      // (a warp beyond the last stick reads nothing: l0 may lie past the table's end)
+      if (nv > 0 && lane <= nv) wd[lane] = __ldg(runs + (long long)k * (nsm + 1) + l0 + lane);
       for (int e = lane; e < Z::LW * Z::S; e += 32) ws[e] = czero<T>();
       __syncwarp();
       if (nv > 0) {
@@ -621,7 +622,7 @@ __global__ void __launch_bounds__(kZThreads)
       const int l0 = blockIdx.x * LPB + (threadIdx.x >> 5) * Z::LW;
       const int nv = min(max(__ldg(nst + k) - l0, 0), Z::LW);
       int4 *wd = zd[threadIdx.x >> 5];
-      if (lane <= nv) wd[lane] = __ldg(runs + (long long)k * (nsm + 1) + l0 + lane);
+      if (nv > 0 && lane <= nv) wd[lane] = __ldg(runs + (long long)k * (nsm + 1) + l0 + lane);
       __syncwarp();
       if (nv == 0) return;
       const int g1 = wd[nv].x;
