@@ -175,7 +175,9 @@ __global__ void __launch_bounds__(256) fft_axis_kernel(cx<T> *__restrict__ data,
   if (MODE == AXIS_FILTER) {
     for (int e = threadIdx.x; e < total; e += blockDim.x) {
       const int j = e / TL, l = e - j * TL;
-      if (l < nlines) in[j * P + l] = cscale<T>(in[j * P + l], io.fac[j * S + i0 + l]);
+      // S == 1 (a grid of one line): the tile's lines are batches, which share the factors
+      if (l < nlines)
+        in[j * P + l] = cscale<T>(in[j * P + l], io.fac[S == 1 ? j : j * S + i0 + l]);
     }
     __syncthreads();
     in = tile_stages<T, TL>(in, in == buf0 ? buf1 : buf0, n, st, tw, +1);
