@@ -191,7 +191,8 @@ tdlz_status tdlz_apply_liouvillian(tdlz_ctx *ctx, int qslot, const void *x, void
 tdlz_status tdlz_chain_create(tdlz_ctx *ctx, const tdlz_lanczos_params *p, tdlz_chain **out);
 /* Enqueue nsteps steps.  From four steps on, pairs of steps are replayed from a
  * CUDA graph recorded on the context stream at the first such call (the graph is
- * re-recorded when the chain's vector rotation differs from the recorded one);
+ * re-recorded when the chain's vector rotation differs from the recorded one, or a larger
+ * chain set on the q-slot has replaced the workspace it points at);
  * results are identical to eager steps.  The caller must not capture the context
  * stream around this call.  With profiling on, every step runs eagerly. */
 tdlz_status tdlz_chain_advance(tdlz_chain *ch, int nsteps);

@@ -105,6 +105,7 @@ template <class T> struct Workspace {
   DevBuf i2;    // staged pipeline without slab stages: [rows][nplane_max][n2][n3] plane scratch
   int nvec_cap = 0;  // stacked vectors the buffers above are sized for
   int ns_cap = 1;    // staged pipeline: vectors per sub-batch its grids are sized for
+  unsigned long long built = 0;  // times the buffers were allocated: recorded graphs hold them
   bool ready = false;
 };
 

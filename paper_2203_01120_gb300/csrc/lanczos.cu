@@ -771,10 +771,15 @@ ChainSet::~ChainSet() {
   if (gexec) cudaGraphExecDestroy(gexec);
 }
 
-std::vector<void *> ChainSet::slot_key() const {
-  std::vector<void *> k;
-  for (const Group &g : groups)
-    for (int i = 0; i < 4; ++i) k.push_back(g.slot[i]);
+// What a recorded graph points at: the vector slots and the q-slots' workspaces, which a
+// larger chain set on the same q-slot replaces.
+std::vector<uintptr_t> ChainSet::graph_state() const {
+  std::vector<uintptr_t> k;
+  for (const Group &g : groups) {
+    for (int i = 0; i < 4; ++i) k.push_back(reinterpret_cast<uintptr_t>(g.slot[i]));
+    const QSlot &s = *ctx->slots[g.qslot];
+    k.push_back((uintptr_t)(precision == TDLZ_FP64 ? s.w64.built : s.w32.built));
+  }
   return k;
 }
 
@@ -810,7 +815,7 @@ void ChainSet::capture_two_steps() {
     gexec = nullptr;
     throw Error{TDLZ_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e)};
   }
-  graph_key = slot_key();
+  graph_key = graph_state();
 }
 
 // Steps run eagerly (one launch sequence per step) while the profiler records
@@ -829,7 +834,7 @@ void ChainSet::advance(int nsteps) {
   for (const Group &g : groups) room = std::min(room, cap - g.host_step);
   const int pairs = room / 2;
   if (pairs > 0) {
-    if (!gexec || graph_key != slot_key()) {
+    if (!gexec || graph_key != graph_state()) {
       NvtxRange cap_range("tdlz/capture");
       capture_two_steps();
     }

@@ -48,9 +48,9 @@ struct ChainSet {
   std::vector<Group> groups;
   DevBuf red;
   // Two steps captured as one CUDA graph (the vector-slot rotation has period 2) and
-  // replayed; valid while the slot arrangement equals the captured one.
+  // replayed; valid while the slots and the q-slots' workspaces are those recorded.
   cudaGraphExec_t gexec = nullptr;
-  std::vector<void *> graph_key;  // slot pointers of every group at capture
+  std::vector<uintptr_t> graph_key;  // graph_state() at capture
   long long graph_kernels = 0;    // kernels in the captured graph
   bool use_graphs = true;
   ~ChainSet();
@@ -67,7 +67,7 @@ struct ChainSet {
   template <class T> void init_impl();
   template <class T> void advance_impl(int nsteps);
   void advance_eager(int nsteps);
-  std::vector<void *> slot_key() const;
+  std::vector<uintptr_t> graph_state() const;
   void capture_two_steps();
 };
 

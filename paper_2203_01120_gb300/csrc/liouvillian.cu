@@ -771,6 +771,7 @@ void alloc_workspace(QSlot &s, int nvec) {
   if (w.ready && w.nvec_cap >= nvec) return;
   const size_t c = sizeof(cx<T>), nv = (size_t)nvec;
   w.ready = false;
+  ++w.built;
   const bool planes = sizeof(T) == 4 ? s.planes32 : s.planes64;
   // fused plane stages: no real-space grids or plane buffer in HBM, only the stick
   // buffer, per-chunk partial densities and the potential planes
