@@ -386,7 +386,10 @@ TnShape tn_shape(int M, int N, long long K, int batch) {
     c.ty = (um + c.ntm - 1) / c.ntm;
     c.tx = (un + c.ntn - 1) / c.ntn;
     const double warps = (double)batch * c.ntm * c.ntn * ((c.ty * c.tx + 31) / 32);
-    for (c.nsplit = 1; c.nsplit <= 32 && (c.nsplit == 1 || K / c.nsplit >= KC); c.nsplit *= 2) {
+    // batch * nsplit is the grid's z extent
+    for (c.nsplit = 1; c.nsplit <= 32 && (c.nsplit == 1 || (K / c.nsplit >= KC &&
+                                                             (long long)batch * c.nsplit <= 65535));
+         c.nsplit *= 2) {
       const double kch = (double)((K + c.nsplit - 1) / c.nsplit);
       // staging and shared-memory loads per product fall with the register tile
       const double t = fp64_clocks(warps * c.nsplit, 4.0 * c.rm * c.rn * kch) *
