@@ -29,7 +29,9 @@
  * input is rejected before any launch.  There is no CPU fallback: without a
  * usable GPU every call fails with TDLZ_ERR_CUDA.  Device work is enqueued on
  * the context's stream; asynchronous faults surface at the next synchronising
- * call (tdlz_synchronize, tdlz_chain_read, tdlz_lanczos_run, tdlz_spectrum).
+ * call (tdlz_synchronize, tdlz_chain_create, tdlz_chain_read, tdlz_chain_save,
+ * tdlz_lanczos_run, tdlz_spectrum).  TDLZ_ERR_TIMEOUT comes from all of these but
+ * tdlz_spectrum, and only on the context whose work it concerns.
  * A context is used by one host thread at a time.
  */
 #ifndef TDLZ_H

@@ -100,6 +100,14 @@ tdlz_status tdlz_create(tdlz_ctx **out, int device, void *cuda_stream) {
     }
     ctx->c.own_stream = true;
   }
+  const tdlz_status st = guarded(ctx, [&] {
+    ctx->c.tc_expired.alloc(sizeof(int));
+    TDLZ_CUDA_TRY(cudaMemsetAsync(ctx->c.tc_expired.p, 0, sizeof(int), ctx->c.stream));
+  });
+  if (st != TDLZ_OK) {
+    tdlz_destroy(ctx);
+    return st;
+  }
   *out = ctx;
   return TDLZ_OK;
 }
@@ -185,8 +193,7 @@ tdlz_status tdlz_autotune_report(tdlz_ctx *ctx, char *buf, int64_t len, int64_t 
 
 tdlz_status tdlz_synchronize(tdlz_ctx *ctx) {
   return guarded(ctx, [&] {
-    TDLZ_CUDA_TRY(cudaStreamSynchronize(ctx->c.stream));
-    tc_gemm_check();
+    tc_gemm_check(ctx->c);
   });
 }
 

@@ -179,6 +179,7 @@ struct Context {
   Profiler prof;
   Tuner tuner;
   DevBuf spec_ws;  // tdlz_spectrum: inputs and chi of the largest call so far
+  DevBuf tc_expired;  // int: a bounded wait of a tensor-core kernel ran out (tc_gemm_check)
 };
 
 template <class T> inline SlotData<T> &slot_data(QSlot &s) {

@@ -850,8 +850,7 @@ void ChainSet::advance(int nsteps) {
 }
 
 void ChainSet::read(tdlz_lanczos_result *res) {
-  TDLZ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-  tc_gemm_check();
+  tc_gemm_check(*ctx);
   for (size_t c = 0; c < chains.size(); ++c) {
     Chain &ch = chains[c];
     ChainScalars hs;
@@ -918,7 +917,7 @@ size_t ChainSet::state_bytes() const {
 
 void ChainSet::save(void *host, size_t bytes) {
   TDLZ_REQUIRE(bytes >= state_bytes(), TDLZ_ERR_ARG, "restart buffer too small");
-  TDLZ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  tc_gemm_check(*ctx);  // no image of vectors that an expired wait spoilt
   char *p = static_cast<char *>(host);
   RestartHeader h{};
   std::memcpy(h.magic, "TDLZRST", 8);

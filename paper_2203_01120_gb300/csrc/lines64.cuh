@@ -49,6 +49,7 @@ struct LineArgs {
   int nl, st, tpr;   // lines per row, bytes between a line's elements (both sides), tiles per row
   long long sp, sf;  // row strides, packed and full side
   long long tiles;
+  int *expired;      // the context's flag: a wait ran out
 };
 
 // fixed point of v, 57 bits below 2^(e - 1022)
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) line_kernel(const LineArgs g) {
       asm volatile("bar.sync 1, %0;" ::"n"(kOzSplit) : "memory");
       ok = __all_sync(0xffffffffu, ok && !bad);
       results(u - 1);
-      if (!ok && lane == 0) atomicExch(&g_tc_timeout, 1);
+      if (!ok && lane == 0) atomicExch(g.expired, 1);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");

@@ -1573,7 +1573,7 @@ void start_vectors(Context &ctx, QSlot &s, const int *mu, int m, cx<T> *v, doubl
       TDLZ_LAUNCH_CHECK();
     }
   }
-  TDLZ_CUDA_TRY(cudaStreamSynchronize(st));
+  tc_gemm_check(ctx);  // (waits for the stream)
 }
 
 // caller order <-> internal order of one BR vector: out[row][i] = in[row][idx[k][i]]

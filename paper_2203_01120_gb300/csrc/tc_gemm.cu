@@ -47,7 +47,6 @@ constexpr int kRowStep = kTcThreads / kChunks;  // rows staged per pass (64)
 constexpr int kMaxA = 64 / kRowStep;            // A rows per thread (M <= 64)
 constexpr int kMaxB = 256 / kRowStep;           // B rows per thread (N tile <= 256)
 
-__device__ int g_tc_timeout = 0;
 __device__ int g_tc_inject = 0;  // test hook: expiries to report after real completion
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -142,6 +141,7 @@ struct TcArgs {
   uint32_t tmem_cols;
   float *part;     // [nsplit][amod][ntiles][128][nt]; transposed form [..][128][nm]
   int nm;          // transposed form: the MMA's N, 2M rounded up to 16
+  int *expired;    // the context's flag: a wait ran out
 };
 
 __global__ void __launch_bounds__(kTcThreads, 2) tc_gemm_tn_kernel(const TcArgs g) {
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_gemm_tn_kernel(const TcArgs 
   quiesce(mbar, abort_flag, abort_it, nloc);
   asm volatile("tcgen05.fence::after_thread_sync;");
   const bool ok = !abort_flag && nloc > 0;
-  if (!ok && tid == 0 && abort_flag) atomicExch(&g_tc_timeout, 1);
+  if (!ok && tid == 0 && abort_flag) atomicExch(g.expired, 1);
   // epilogue: warp w reads TMEM lanes (rows) 32 (w & 3) .. + 31 (its lane quarter),
   // the two warps of a quarter take alternate 8-column chunks
   const int quarter = warp & 3;
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_gemm_tnt_kernel(const TcArgs
   quiesce(mbar, abort_flag, abort_it, nloc);
   asm volatile("tcgen05.fence::after_thread_sync;");
   const bool ok = !abort_flag && nloc > 0;
-  if (!ok && tid == 0 && abort_flag) atomicExch(&g_tc_timeout, 1);
+  if (!ok && tid == 0 && abort_flag) atomicExch(g.expired, 1);
   // epilogue: warp w reads TMEM lanes 32 (w & 3) .. + 31 (stacked rows R), the two warps
   // of a quarter take alternate 8-column chunks of the nm columns
   const int quarter = warp & 3;
@@ -587,6 +587,7 @@ struct NnArgs {
   float alpha;
   int neg_from, neg_mod;
   uint32_t tmem_cols;
+  int *expired;    // the context's flag: a wait ran out
 };
 
 __global__ void __launch_bounds__(kTcThreads, 2) tc_gemm_nn_kernel(const NnArgs g) {
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_gemm_nn_kernel(const NnArgs 
   quiesce(mbar, abort_flag, abort_it, g.nkt);
   asm volatile("tcgen05.fence::after_thread_sync;");
   const bool ok = !abort_flag;
-  if (abort_flag && tid == 0) atomicExch(&g_tc_timeout, 1);
+  if (abort_flag && tid == 0) atomicExch(g.expired, 1);
   // epilogue: warp w reads lane quarter w & 3 (32 consecutive columns n); the two warps
   // of a quarter take alternate 16-column TMEM blocks (8 output rows each)
   const int quarter = warp & 3;
@@ -775,6 +776,7 @@ bool tc_gemm_tn_transposed(Context &ctx, DevBuf &partbuf, const float2 *A, long 
                            float2 *C, long long sC, long long ldcm, long long ldcn, int M, int N,
                            long long K, int batch) {
   TcArgs g{};
+  g.expired = ctx.tc_expired.as<int>();
   g.A = A;
   g.lda = lda;
   g.sA = sA;
@@ -944,6 +946,7 @@ struct NnImgArgs {
   float alpha;
   int neg_from, neg_mod;
   uint32_t tmem_cols, in_bytes, stage_bytes;
+  int *expired;    // the context's flag: a wait ran out
 };
 
 // One CTA per (batch b, 128-column tile); the CTAs of the batches b = g + j G that share
@@ -1083,7 +1086,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
   __syncthreads();
   const bool ok = !abort_flag && n_commit == g.nkt;
-  if (tid == 0 && abort_flag) atomicExch(&g_tc_timeout, 1);
+  if (tid == 0 && abort_flag) atomicExch(g.expired, 1);
   if (ok) {
     // completed phases: these waits return at once and order the MMAs' TMEM writes and
     // the tensor copy's shared-memory writes before this thread's reads
@@ -1212,6 +1215,7 @@ bool tc_gemm_tn(Context &ctx, DevBuf &partbuf, const float2 *A, long long lda, l
     return tc_gemm_tn_transposed(ctx, partbuf, A, lda, sA, amod, B, ldb, sB, C, sC, ldcm, ldcn,
                                  M, N, K, batch);
   TcArgs g;
+  g.expired = ctx.tc_expired.as<int>();
   g.A = A;
   g.lda = lda;
   g.sA = sA;
@@ -1272,6 +1276,7 @@ bool tc_gemm_nn(Context &ctx, const float2 *A, long long sA, long long sar, long
     return true;
   }
   NnArgs g;
+  g.expired = ctx.tc_expired.as<int>();
   g.A = A;
   g.sA = sA;
   g.sar = sar;
@@ -1364,6 +1369,7 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
   for (int r0 = 0; r0 < rows; r0 += R) {
     const int nr = std::min(R, rows - r0);
     NnImgArgs g{};
+    g.expired = ctx.tc_expired.as<int>();
     g.aimg = im.buf.as<unsigned char>();
     g.bimg = scratch.as<unsigned char>();
     g.In = In + (long long)r0 * ldo;
@@ -1445,6 +1451,7 @@ bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda
                   long long K, int batch, double clocks, double2 *&part, int &nsplit) {
   if (batch % amod != 0 || K < 64) return false;
   OzArgs g{};
+  g.expired = ctx.tc_expired.as<int>();
   g.A = A;
   g.lda = lda;
   g.sA = sA;
@@ -1504,6 +1511,7 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
                   long long ncol, int K, double alpha, int batch, int neg_from, int neg_mod,
                   double clocks) {
   OzArgs g{};
+  g.expired = ctx.tc_expired.as<int>();
   g.A = A;
   g.sA = sA;
   g.sar = sar;
@@ -1642,6 +1650,7 @@ bool tc_lines(Context &ctx, QSlot &s, int axis, bool inverse, const double2 *src
               long long rows) {
   if (!tc_lines_taken(s, axis)) return false;
   LineArgs g{};
+  g.expired = ctx.tc_expired.as<int>();
   const long long n2 = s.fft[1], n3 = s.fft[2];
   g.src = src;
   g.dst = dst;
@@ -1679,12 +1688,13 @@ void tc_gemm_inject_timeout(int n) {
   TDLZ_CUDA_TRY(cudaMemcpyToSymbol(g_tc_inject, &n, sizeof(int)));
 }
 
-void tc_gemm_check() {
+void tc_gemm_check(Context &ctx) {
   int flag = 0;
-  TDLZ_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_tc_timeout, sizeof(int)));
+  int *p = ctx.tc_expired.as<int>();
+  TDLZ_CUDA_TRY(cudaMemcpyAsync(&flag, p, sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
+  TDLZ_CUDA_TRY(cudaStreamSynchronize(ctx.stream));
   if (flag) {
-    int zero = 0;
-    TDLZ_CUDA_TRY(cudaMemcpyToSymbol(g_tc_timeout, &zero, sizeof(int)));
+    TDLZ_CUDA_TRY(cudaMemsetAsync(p, 0, sizeof(int), ctx.stream));
     throw Error{TDLZ_ERR_TIMEOUT, "tensor-core GEMM: an mbarrier wait ran out (results invalid)"};
   }
 }

@@ -68,9 +68,9 @@ bool tc_lines_taken(const QSlot &s, int axis);
 // n > 48, h > 15, 2 h >= n, or sums beyond the accumulators' exact range.
 bool tc_lines_build(int n, int h, std::vector<uint16_t> &img);
 
-// Throws TDLZ_ERR_TIMEOUT (and clears the flag) if a tensor-core GEMM gave up on an
-// mbarrier wait since the last check.  Synchronous.
-void tc_gemm_check();
+// Waits for the context's stream; throws TDLZ_ERR_TIMEOUT (and clears the context's flag) if
+// a tensor-core kernel of this context gave up on an mbarrier wait since the last check.
+void tc_gemm_check(Context &ctx);
 
 // Test hook (TDLZ_TEST_INJECT_TC_TIMEOUT=n at context creation): the next n bounded
 // mbarrier waits that complete report expiry instead, so that the abort path runs (and

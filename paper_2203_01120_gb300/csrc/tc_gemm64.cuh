@@ -76,6 +76,7 @@ struct OzArgs {
   long long ldo, sO;
   double alpha;
   int neg_from, neg_mod;
+  int *expired;      // the context's flag: a wait ran out
 };
 
 // max biased exponent of rows of len complex elements: row r starts at
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
       ok = __all_sync(0xffffffffu, ok && !bad);
       drain();
       output(t1 - 1);
-      if (!ok && lane == 0) atomicExch(&g_tc_timeout, 1);
+      if (!ok && lane == 0) atomicExch(g.expired, 1);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
