@@ -33,6 +33,13 @@
  * tdlz_lanczos_run, tdlz_spectrum).  TDLZ_ERR_TIMEOUT comes from all of these but
  * tdlz_spectrum, and only on the context whose work it concerns.
  * A context is used by one host thread at a time.
+ *
+ * TDLZ_FP64 stores and returns doubles.  Larger X and Y lines and contractions (V_NL, P_c,
+ * the start vectors of either precision) run as exact integer products of fixed-point rows
+ * on the tensor cores: lines 57 bits below their largest element, contractions 62 bits, with
+ * every output whose sum of magnitudes is too small for that formed by FP64 multiply-adds
+ * instead.  Errors stay those of FP64 transforms and sums, component by component.  A row or
+ * line with a non-finite element gives NaN where FP64 arithmetic might give an infinity.
  */
 #ifndef TDLZ_H
 #define TDLZ_H

@@ -829,7 +829,18 @@ void alloc_workspace(QSlot &s, int nvec) {
       p3 = std::max(p3, 32 * groups * tiles * 128 *
                             (((cols + tiles - 1) / tiles + 15) / 16 * 16) * sizeof(float));
     }
-  w.part.alloc(std::max(std::max(p1, p2) * c, p3));
+  // FP64 slices: their rows' exponents and norms (both contractions) beside the partial sums
+  size_t p4 = 0, p5 = 0;
+  if (sizeof(T) == 8 && s.tensor_gemm) {
+    const int nk = s.nk, nb = s.nb, b = (int)batch;
+    p4 = tc_gemm64_tn_scratch(2 * nk, nb, b, nb, 32);
+    p5 = tc_gemm64_nn_scratch(b, nb, 2 * nk, 2LL * s.npwx);
+    if (s.nproj > 0) {
+      p4 = std::max(p4, tc_gemm64_tn_scratch(nk, s.nproj, b, 2 * nb, 32));
+      p5 = std::max(p5, tc_gemm64_nn_scratch(b, 2 * nb, nk, s.npwx));
+    }
+  }
+  w.part.alloc(std::max({std::max(p1, p2) * c + p4, p3, p5}));
   w.nvec_cap = nvec;
   w.ready = true;
 }
@@ -1540,14 +1551,15 @@ void start_vectors(Context &ctx, QSlot &s, const int *mu, int m, cx<T> *v, doubl
   const long long bstride = (long long)nb * 2 * npwx, br = s.br_elems();
   DevBuf ovb, partb;
   ovb.alloc((size_t)most * batch1 * nb * nb * sizeof(double2));
-  // K splits: the FP64-pipe form's, or a tile of the slices per SM; row exponents of the slices
+  // K splits: the FP64-pipe form's, or a tile of the slices per SM, with the slices' row scales
   const int last = m % most ? m % most : most;
   const int splits = std::max({tn_shape(nb, nb, 2LL * npwx, most * batch1).nsplit,
                                tn_shape(nb, nb, 2LL * npwx, last * batch1).nsplit,
                                std::min(32, 1 + 152 / batch1)});
   const size_t outs = (size_t)most * batch1 * nb * nb;
-  partb.alloc(splits * outs * sizeof(double2) +
-              ((size_t)(most + 1) * batch1 * (nb + 2LL * npwx) + 64) * sizeof(int));
+  partb.alloc(std::max(splits * outs * sizeof(double2) +
+                           tc_gemm64_tn_scratch(batch1, nb, most * batch1, nb, splits),
+                       tc_gemm64_nn_scratch(most * batch1, nb, batch1, 2LL * npwx)));
   double2 *ov = ovb.as<double2>();
   const double2 *ukq = s.d64.ukq.as<double2>();
   for (int c0 = 0; c0 < m; c0 += most) {

@@ -1432,19 +1432,61 @@ void oz_tiles(OzArgs &g) {
   g.mt = (g.M + g.ntn - 1) / g.ntn;
   g.nt = (2 * g.mt + 15) / 16 * 16;
 }
+long long oz_row_tiles(long long rows) { return (rows + 127) / 128; }
 
 template <bool NN> void oz_launch(Context &ctx, const OzArgs &g) {
   // two stages and the raw elements; at least 116 KB: one CTA per SM (it takes all of TMEM)
-  const size_t smem = 2ull * kOzS * (kOzATile + (size_t)g.nt * kOzKT * 2) +
-                      16ull * 4 * (kOzSplit + 2 * kOzMaxNt);
+  const size_t smem = 2ull * oz_stage(g.nt, g.mt) + 16ull * 4 * (kOzSplit + 2 * kOzMaxNt);
   const size_t ask = std::max(smem, (size_t)116 * 1024);
   TDLZ_CUDA_TRY(cudaFuncSetAttribute(oz_gemm_kernel<NN>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ask));
   oz_gemm_kernel<NN><<<(unsigned)std::min(152LL, g.tiles), kOzThreads, ask, ctx.stream>>>(g);
   TDLZ_LAUNCH_CHECK();
+  oz_redo_kernel<NN><<<(unsigned)std::min(8 * 152LL, 4 * g.tiles), 128, 0, ctx.stream>>>(g);
+  TDLZ_LAUNCH_CHECK();
 }
 
+// Scratch of rows' exponents, norms and bits and tiles' flags, in front of the partial sums.
+struct OzScratch {
+  size_t ea, eb, na, nb, ba, bb, redo, bytes;
+  OzScratch(long long ra, long long rb, long long tiles) {
+    ba = 0;
+    bb = ba + 32 * (size_t)ra;
+    ea = bb + 32 * (size_t)rb;
+    eb = ea + 4 * (size_t)ra;
+    na = eb + 4 * (size_t)rb;
+    nb = na + 4 * (size_t)ra;
+    redo = (nb + 4 * (size_t)rb + 15) & ~(size_t)15;
+    bytes = (redo + 16 * (size_t)tiles + 255) & ~(size_t)255;
+  }
+  void set(OzArgs &g, char *p) const {
+    g.ea = reinterpret_cast<int *>(p + ea);
+    g.eb = reinterpret_cast<int *>(p + eb);
+    g.na = reinterpret_cast<float *>(p + na);
+    g.nb = reinterpret_cast<float *>(p + nb);
+    g.ba = reinterpret_cast<uint4 *>(p + ba);
+    g.bb = reinterpret_cast<uint4 *>(p + bb);
+    g.redo = reinterpret_cast<unsigned char *>(p + redo);
+  }
+};
+
 }  // namespace
+
+size_t tc_gemm64_tn_scratch(int amod, int M, int batch, int N, int nsplit) {
+  OzArgs g{};
+  g.M = M;
+  oz_tiles(g);
+  const long long tiles = oz_row_tiles((long long)(batch / amod) * N) * g.ntn * amod;
+  return OzScratch((long long)amod * M * nsplit, (long long)batch * N * nsplit, tiles * nsplit)
+      .bytes;
+}
+
+size_t tc_gemm64_nn_scratch(int batch, int rows, int bmod, long long ncol) {
+  OzArgs g{};
+  g.M = rows;
+  oz_tiles(g);
+  return OzScratch((long long)batch * rows, bmod * ncol, oz_row_tiles(ncol) * g.ntn * batch).bytes;
+}
 
 bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda, long long sA,
                   int amod, const double2 *B, long long ldb, long long sB, int M, int N,
@@ -1465,41 +1507,46 @@ bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda
   g.batch = batch;
   g.nj = batch / amod;
   g.ntot = g.nj * N;
-  g.ntm = (g.ntot + 127) / 128;
+  g.ntm = (int)oz_row_tiles(g.ntot);
   oz_tiles(g);
   const long long nst = (K + kOzKT / 2 - 1) / (kOzKT / 2);
   const long long tiles = (long long)g.ntm * g.ntn * amod;
-  const size_t nexp = ((size_t)amod * M + (size_t)batch * N) * sizeof(int);
-  const size_t off = (nexp + 255) & ~(size_t)255, one = (size_t)batch * M * N * sizeof(double2);
-  if (partbuf.bytes < off + one) return false;
+  const long long ra = (long long)amod * M, rb = (long long)batch * N;
+  const size_t one = (size_t)batch * M * N * sizeof(double2);
   // K splits of whole drains, within the scratch: the number whose tiles the CTAs walk soonest
   // (96 tiles of 1500 stages, one split: 1500 stage times; three: 1000)
   long long kst = 0;
   double best = 0.0;
-  const long long most = std::min({(nst + 3) / 4, (long long)((partbuf.bytes - off) / one), 64LL});
-  for (long long ns = 1; ns <= most; ++ns) {
+  for (long long ns = 1; ns <= std::min((nst + 3) / 4, 64LL); ++ns) {
     const long long st = ((nst + ns - 1) / ns + kOzDrain - 1) / kOzDrain * kOzDrain;
-    const double t = oz_clocks((double)tiles * ((nst + st - 1) / st), (double)st, g.nt);
+    const long long n = (nst + st - 1) / st;
+    if (OzScratch(ra * n, rb * n, tiles * n).bytes + n * one > partbuf.bytes) break;
+    const double t = oz_clocks((double)tiles * n, (double)st, g.nt);
     if (kst == 0 || t < best) {
       best = t;
       kst = st;
     }
   }
+  if (kst == 0) return false;
   g.kst = (int)kst;
   g.nsplit = (int)((nst + kst - 1) / kst);
   g.tiles = tiles * g.nsplit;
   if (kst > 1 << 16) return false;  // 2^14 drains: the sums stay below 2^63
   if (best > 0.7 * clocks) return false;
-  int *e = partbuf.as<int>();
-  g.ea = e;
-  g.eb = e + (size_t)amod * M;
-  part = reinterpret_cast<double2 *>(partbuf.as<char>() + off);
+  const OzScratch sc(ra * g.nsplit, rb * g.nsplit, g.tiles);
+  sc.set(g, partbuf.as<char>());
+  g.rk = std::sqrt((float)(kst * kOzKT));
+  part = reinterpret_cast<double2 *>(partbuf.as<char>() + sc.bytes);
   g.part = part;
   nsplit = g.nsplit;
-  const long long ra = (long long)amod * M, rb = (long long)batch * N;
-  oz_row_exp_kernel<<<(unsigned)ra, 128, 0, ctx.stream>>>(A, M, sA, lda, 1, K, e);
+  const long long kc = kst * (kOzKT / 2);
+  oz_row_scale_kernel<<<dim3((unsigned)ra, nsplit), 128, 0, ctx.stream>>>(
+      A, M, sA, lda, 1, K, kc, const_cast<int *>(g.ea), const_cast<float *>(g.na),
+      (uint32_t *)g.ba);
   TDLZ_LAUNCH_CHECK();
-  oz_row_exp_kernel<<<(unsigned)rb, 128, 0, ctx.stream>>>(B, N, sB, ldb, 1, K, e + ra);
+  oz_row_scale_kernel<<<dim3((unsigned)rb, nsplit), 128, 0, ctx.stream>>>(
+      B, N, sB, ldb, 1, K, kc, const_cast<int *>(g.eb), const_cast<float *>(g.nb),
+      (uint32_t *)g.bb);
   TDLZ_LAUNCH_CHECK();
   oz_launch<false>(ctx, g);
   return true;
@@ -1534,17 +1581,21 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
   oz_tiles(g);
   g.nsplit = 1;
   g.kst = (K + kOzKT / 2 - 1) / (kOzKT / 2);
-  g.ntm = (int)((ncol + 127) / 128);
+  g.ntm = (int)oz_row_tiles(ncol);
   g.tiles = (long long)g.ntm * g.ntn * batch;
   if (oz_clocks((double)g.tiles, (double)g.kst, g.nt) > 0.7 * clocks) return false;
   const long long ra = (long long)batch * rows, cb = (long long)bmod * ncol;
-  if (scratch.bytes < (size_t)(ra + cb) * sizeof(int)) return false;
-  int *e = scratch.as<int>();
-  g.ea = e;
-  g.eb = e + ra;
-  oz_row_exp_kernel<<<(unsigned)ra, 128, 0, ctx.stream>>>(A, rows, sA, sar, sak, K, e);
+  const OzScratch sc(ra, cb, g.tiles);
+  if (scratch.bytes < sc.bytes) return false;
+  sc.set(g, scratch.as<char>());
+  g.rk = std::sqrt(2.f * K);
+  oz_row_scale_kernel<<<(unsigned)ra, 128, 0, ctx.stream>>>(
+      A, rows, sA, sar, sak, K, K, const_cast<int *>(g.ea), const_cast<float *>(g.na),
+      (uint32_t *)g.ba);
   TDLZ_LAUNCH_CHECK();
-  oz_col_exp_kernel<<<blocks_for(cb), 256, 0, ctx.stream>>>(B, ldb, sB, bmod, K, ncol, e + ra);
+  oz_col_scale_kernel<<<blocks_for(cb), 256, 0, ctx.stream>>>(
+      B, ldb, sB, bmod, K, ncol, const_cast<int *>(g.eb), const_cast<float *>(g.nb),
+      (uint32_t *)g.bb);
   TDLZ_LAUNCH_CHECK();
   oz_launch<true>(ctx, g);
   return true;

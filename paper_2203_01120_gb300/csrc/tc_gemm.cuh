@@ -43,10 +43,10 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
 
 // FP64 contractions by exact integer slices on the tensor cores (tc_gemm64.cuh), where their
 // estimated clocks are below 0.7 of `clocks`, the estimate of the FP64-pipe form; otherwise
-// false, launching nothing.  The reduction writes its partial sums
-// part[z][b][m][n], z < nsplit, behind the row exponents in partbuf; the update needs
-// (batch rows + bmod ncol) ints of scratch.  Same contracts as tc_gemm_tn and tc_gemm_nn; a
-// row with a non-finite element gives NaN.
+// false, launching nothing.  Outputs for which 62-bit rows could cost more than the rounding of
+// an FP64 sum are formed by FP64 multiply-adds.  The reduction writes its partial sums
+// part[z][b][m][n], z < nsplit, behind its scratch in partbuf.  Same contracts as tc_gemm_tn
+// and tc_gemm_nn; a row with a non-finite element gives NaN.
 bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda, long long sA,
                   int amod, const double2 *B, long long ldb, long long sB, int M, int N,
                   long long K, int batch, double clocks, double2 *&part, int &nsplit);
@@ -55,6 +55,9 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
                   const double2 *In, double2 *Out, long long ldo, long long sO, int rows,
                   long long ncol, int K, double alpha, int batch, int neg_from, int neg_mod,
                   double clocks);
+// Scratch of the two without the partial sums (rows' exponents and norms, tiles' flags).
+size_t tc_gemm64_tn_scratch(int amod, int M, int batch, int N, int nsplit);
+size_t tc_gemm64_nn_scratch(int batch, int rows, int bmod, long long ncol);
 
 // X (axis 0) or Y (axis 1) line transforms of the FP64 pipeline on the tensor cores
 // (lines64.cuh), between its packed and full buffers (inverse: packed to full).  Returns false,

@@ -8,11 +8,27 @@
 // pairs (i, j) with i + j = D over 128 terms exactly (8 x 128 x 2^14 = 2^24).  Eight
 // accumulators, D = 0..7 (36 of the 64 pairs; the rest lie 2^-62 below the rows' largest
 // products), sit side by side in TMEM; every 128 terms they are drained into two 64-bit
-// integers per output, and only the last step is FP64.  Nothing is rounded in between:
-// the error is the 62-bit quantisation of the rows, below the rounding of an FP64 sum unless
-// a row's largest element lies more than a factor of 2^9 above its typical one (the error-free
-// splitting of T. Ozaki, K. Ogita, S. Oishi, S. Rump, Numer. Algorithms 59,
-// 2012; on integer-valued tensor-core sums: Mukunoki et al., ISC 2020).
+// integers per output, and only the last step is FP64 (the error-free splitting of T. Ozaki,
+// K. Ogita, S. Oishi, S. Rump, Numer. Algorithms 59, 2012; on integer-valued tensor-core
+// sums: Mukunoki et al., ISC 2020).
+//
+// What is lost are bits 2^-62 below a row's largest element: nothing beside the rounding of an
+// FP64 sum where the products that matter are formed by elements near the rows' largest, but
+// all of it where large elements of one row meet small ones of the other (a projector that
+// falls over 17 decades, a vector that grows by 10^6 over the same plane waves: 1e-12 of the
+// result instead of 2e-16).  Each output is therefore tested, with quantities of its own:
+// with the rows scaled by their powers of two, its error is about
+//   2^-62 (||a|| + ||b|| + sqrt(K)),   K real terms,
+// (truncated elements, left-out digit pairs), an FP64 sum's about 2^-53 S, S = sum |a_k| |b_k|.
+// S comes from one more MMA per stage, of the two leading digits' magnitudes rounded down to
+// E5M2, the norms from the pass that finds the exponents.  Where
+//   S < 2^-9 (||a|| + ||b|| + sqrt(K))
+// and the two rows' nonzero elements meet at all (256 bits per row, OzBits; states of opposite
+// spins don't) and, in the update, the addend is as small, a second
+// kernel forms the outputs of that warp's 32 x nt / 8 block by FP64 multiply-adds
+// (oz_redo_kernel).  Against exact sums (the integer steps on the host, 300 to 2400 terms,
+// flat, Gaussian, sparse and growing rows) outputs that pass have errors of at most
+// 0.9 2^-53 S, FP64 sums of the same rows 0.7 to 8.8.
 //
 // One CTA per SM, with all 512 TMEM columns, walks its share of the (output tile of 128 rows x
 // nt <= 48 columns, K split) list, 32 reals of K per stage, two stages: sixteen warps copy the
@@ -69,7 +85,11 @@ struct OzArgs {
   long long lda, sA, ldb, sB, sar, sak;
   int amod, M, N, nj, ntot, ntm, ntn, mt, nt, nsplit, batch, kst;  // kst: stages per split
   long long K, ncol, tiles;
-  const int *ea, *eb;  // row exponents of A and of B (NN: of B's columns)
+  const int *ea, *eb;    // exponents of A's and B's rows per split (NN: of B's columns)
+  const float *na, *nb;  // their 2-norms over 2^(exponent - 1022)
+  const uint4 *ba, *bb;  // which of their elements are not 0, two each (OzBits)
+  float rk;              // square root of a split's real terms
+  unsigned char *redo;   // [tile][16 warps]: block left to oz_redo_kernel
   double2 *part;
   const double2 *In;
   double2 *Out;
@@ -79,42 +99,205 @@ struct OzArgs {
   int *expired;      // the context's flag: a wait ran out
 };
 
-// max biased exponent of rows of len complex elements: row r starts at
-// p + (r / per) s0 + (r % per) s1, elements sk apart; one block per row
-__global__ void __launch_bounds__(128)
-    oz_row_exp_kernel(const double2 *__restrict__ p, int per, long long s0, long long s1,
-                      long long sk, long long len, int *__restrict__ e) {
-  const long long r = blockIdx.x;
-  const double2 *q = p + (r / per) * s0 + (r % per) * s1;
+// Largest biased exponent m (at least 1) of the numbers seen so far and the sum s of their
+// squares over 2^(2 m - 2044), without FP64 instructions.
+struct OzScale {
   int m = 1;
-#pragma unroll 4
-  for (long long k = threadIdx.x; k < len; k += blockDim.x) {
-    const double2 v = q[k * sk];
-    m = max(m, max(oz_exp(v.x), oz_exp(v.y)));
+  float s = 0.f;
+  // 2^(2 d), d <= 0; 0 below the range
+  static __device__ __forceinline__ float pow4(int d) {
+    return d > -63 ? __int_as_float((127 + 2 * d) << 23) : 0.f;
   }
-  __shared__ int sh[4];
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __device__ __forceinline__ void square(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    const int ex = (int)(hi >> 20), x = 126 + ex - m;
+    const float f = ex > 0 && x > 0 ? __int_as_float(x << 23 | (int)((hi & 0xfffffu) << 3)) : 0.f;
+    s = fmaf(f, f, s);
+  }
+  __device__ __forceinline__ void add(double2 v) {
+    const int e = max(oz_exp(v.x), oz_exp(v.y));
+    if (e > m) {
+      s *= pow4(m - e);
+      m = e;
+    }
+    square(v.x);
+    square(v.y);
+  }
+};
+
+// v != 0, by its words (a comparison is an FP64 instruction)
+__device__ __forceinline__ bool oz_nonzero(double2 v) {
+  return (((uint32_t)__double2hiint(v.x) << 1) | (uint32_t)__double2loint(v.x) |
+          ((uint32_t)__double2hiint(v.y) << 1) | (uint32_t)__double2loint(v.y)) != 0;
+}
+
+// Bit of element k of a row of len: its own where len <= 256, else that of its run, 128 equal ones
+// in each half (the halves of a spinor are its spins).
+struct OzBits {
+  uint32_t half, magic;  // of the division by the run's length
+  bool own;
+  __device__ OzBits(long long len) {
+    own = len <= 256;
+    half = (uint32_t)((len + 1) >> 1);
+    magic = 0xffffffffu / ((half + 127) >> 7) + 1u;  // a run of 1: own is set
+  }
+  __device__ __forceinline__ int at(uint32_t k) const {
+    if (own) return (int)k;
+    const bool h = k >= half;
+    return (int)(__umulhi(k - (h ? half : 0u), magic) + (h ? 128u : 0u));
+  }
+};
+__device__ __forceinline__ bool oz_meet(const uint4 *a, const uint4 *b) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint4 x = a[i], y = b[i];
+    m |= (x.x & y.x) | (x.y & y.y) | (x.z & y.z) | (x.w & y.w);
+  }
+  return m != 0;
+}
+
+// exponent, norm and bits of rows of at most kc complex elements, one block per (row, split): row
+// r starts at p + (r / per) s0 + (r % per) s1, elements sk apart, split y at element y kc of len
+__global__ void __launch_bounds__(128)
+    oz_row_scale_kernel(const double2 *__restrict__ p, int per, long long s0, long long s1,
+                        long long sk, long long len, long long kc, int *__restrict__ e,
+                        float *__restrict__ nrm, uint32_t *__restrict__ bits) {
+  const long long r = blockIdx.x, k0 = blockIdx.y * kc, k1 = min(len, k0 + kc);
+  const double2 *q = p + (r / per) * s0 + (r % per) * s1;
+  const OzBits ob(len);
+  const int tid = threadIdx.x;
+  __shared__ int shm[4];
+  __shared__ float shs[4];
+  __shared__ uint32_t shb[8];
+  if (tid < 8) shb[tid] = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, sh[w]);
-    e[r] = m;
+  OzScale a;
+#pragma unroll 4
+  for (long long k = k0 + tid; k < k1; k += 128) {
+    const double2 v = q[k * sk];
+    a.add(v);
+    if (oz_nonzero(v)) {
+      const int b = ob.at((uint32_t)k);
+      if (!(*(volatile uint32_t *)(shb + (b >> 5)) >> (b & 31) & 1u))
+        atomicOr(shb + (b >> 5), 1u << (b & 31));
+    }
+  }
+  const int wm = __reduce_max_sync(0xffffffffu, a.m);
+  if ((tid & 31) == 0) shm[tid >> 5] = wm;
+  __syncthreads();
+  const int m = max(max(shm[0], shm[1]), max(shm[2], shm[3]));
+  float s = a.s * OzScale::pow4(a.m - m);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((tid & 31) == 0) shs[tid >> 5] = s;
+  __syncthreads();
+  const long long at = (long long)blockIdx.y * gridDim.x + r;
+  if (tid < 8) bits[8 * at + tid] = shb[tid];
+  if (tid == 0) {
+    e[at] = m;
+    nrm[at] = sqrtf(shs[0] + shs[1] + shs[2] + shs[3]);
   }
 }
 
-// max biased exponent of the columns n of B[g][k][n], k < K
-__global__ void oz_col_exp_kernel(const double2 *__restrict__ B, long long ldb, long long sB,
-                                  int G, int K, long long ncol, int *__restrict__ e) {
+// exponent, norm and bits of the columns n of B[g][k][n], k < K <= 256
+__global__ void oz_col_scale_kernel(const double2 *__restrict__ B, long long ldb, long long sB,
+                                    int G, int K, long long ncol, int *__restrict__ e,
+                                    float *__restrict__ nrm, uint32_t *__restrict__ bits) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= G * ncol) return;
   const long long g = i / ncol;
   const double2 *q = B + g * sB + (i - g * ncol);
-  int m = 1;
-  for (int k = 0; k < K; ++k) {
-    const double2 v = q[(long long)k * ldb];
-    m = max(m, max(oz_exp(v.x), oz_exp(v.y)));
+  OzScale a;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t m[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int k0 = 128 * h + 32 * w;
+      m[w] = 0;
+#pragma unroll 4
+      for (int k = k0; k < min(K, k0 + 32); ++k) {
+        const double2 v = q[(long long)k * ldb];
+        a.add(v);
+        if (oz_nonzero(v)) m[w] |= 1u << (k & 31);
+      }
+    }
+    reinterpret_cast<uint4 *>(bits)[2 * i + h] = make_uint4(m[0], m[1], m[2], m[3]);
   }
-  e[i] = m;
+  e[i] = a.m;
+  nrm[i] = sqrtf(a.s);
+}
+
+// Magnitudes of four numbers from the FP16 pairs of their two leading digits: 256 d_0 + d_1,
+// 2^14 over the row's scale, rounded down to E5M2 (the upper byte of FP16).
+__device__ __forceinline__ uint32_t oz_mag(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1) {
+  uint32_t a, b;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(a) : "r"(a0), "r"(0x5c005c00u), "r"(a1));
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(b) : "r"(b0), "r"(0x5c005c00u), "r"(b1));
+  return __byte_perm(a, b, 0x7531) & 0x7f7f7f7fu;
+}
+
+// Rows of the column operand's magnitudes (the S MMA's N) and bytes of a stage: digits of the
+// rows, digits of the columns, magnitudes of the rows and of the columns (32 bytes a row each).
+__host__ __device__ constexpr int oz_ns(int mt) { return mt > 16 ? 32 : 16; }
+constexpr uint32_t kOzSTile = 128 * kOzKT;
+__host__ __device__ constexpr uint32_t oz_stage(int nt, int mt) {
+  return kOzS * (kOzATile + (uint32_t)nt * kOzKT * 2) + kOzSTile + (uint32_t)oz_ns(mt) * kOzKT;
+}
+
+// Tile t = ((z ntn + tn) ntm + tm): TN row tile tm of stacked (j, n), column tile tn of m,
+// z = split amod + A batch; NN row tile of columns n, column tile of r, z = batch
+struct OzTile {
+  int tm, tn, a, sp, b, bg, nst;
+  long long kc0;  // first complex k
+};
+template <bool NN> __device__ __forceinline__ OzTile oz_tile(const OzArgs &g, long long t) {
+  OzTile q;
+  q.tm = (int)(t % g.ntm);
+  t /= g.ntm;
+  q.tn = (int)(t % g.ntn);
+  const int z = (int)(t / g.ntn);
+  q.a = NN ? 0 : z % g.amod;
+  q.sp = NN ? 0 : z / g.amod;
+  q.b = NN ? z : 0;
+  q.bg = NN ? z % g.amod : 0;  // NN: amod holds bmod
+  q.kc0 = (long long)q.sp * g.kst * (kOzKT / 2);
+  q.nst = (int)min((long long)g.kst, (g.K - q.kc0 + kOzKT / 2 - 1) / (kOzKT / 2));
+  return q;
+}
+// A tile's row R: batch and index of its row operand, place of its exponent, valid or not.
+struct OzRow {
+  bool in;
+  long long b, n, e;
+};
+template <bool NN>
+__device__ __forceinline__ OzRow oz_row(const OzArgs &g, const OzTile &q, long long R) {
+  OzRow r;
+  if (NN) {
+    r.in = R < g.ncol;
+    r.b = q.b;
+    r.n = R;
+    r.e = q.bg * g.ncol + R;
+  } else {
+    r.in = R < g.ntot;
+    const int j = (int)(R / g.N);
+    r.n = R - (long long)j * g.N;
+    r.b = q.a + (long long)j * g.amod;
+    r.e = ((long long)q.sp * g.batch + r.b) * g.N + r.n;
+  }
+  return r;
+}
+// Place of the exponent of a tile's column cg, and of output (row, column cg).
+template <bool NN>
+__device__ __forceinline__ long long oz_col(const OzArgs &g, const OzTile &q, int cg) {
+  return (NN ? (long long)q.b : (long long)q.sp * g.amod + q.a) * g.M + cg;
+}
+template <bool NN>
+__device__ __forceinline__ long long oz_at(const OzArgs &g, const OzTile &q, const OzRow &r,
+                                           int cg) {
+  return NN ? r.b * g.sO + (long long)cg * g.ldo + r.n
+            : (((long long)q.sp * g.batch + r.b) * g.M + cg) * g.N + r.n;
 }
 
 // (hi 2^32 + lo) 2^e as a double, rounded once, without an FP64 instruction
@@ -170,32 +353,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
   __shared__ int bad;  // a wait expired
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nt = g.nt;
-  const uint32_t bTile = (uint32_t)nt * kOzKT * 2, lboA = 2048;
-  const uint32_t lboB = (uint32_t)(kOzS * nt) * 16;  // the column digits' rows side by side
-  const uint32_t stage_bytes = kOzS * (kOzATile + bTile);
-  // tiles [t0, t1) of this CTA, tile = ((z ntn + tn) ntm + tm): TN row tile tm of stacked
-  // (j, n), column tile tn of m, z = split amod + A batch; NN row tile of columns n, column
-  // tile of r, z = batch
+  const uint32_t lboA = 2048, lboB = (uint32_t)(kOzS * nt) * 16;  // column digits side by side
+  const uint32_t stage_bytes = oz_stage(nt, g.mt), ns = (uint32_t)oz_ns(g.mt);
+  const uint32_t sOff = kOzS * (kOzATile + (uint32_t)nt * kOzKT * 2);  // magnitudes in a stage
+  // tiles [t0, t1) of this CTA
   const long long t0 = g.tiles * blockIdx.x / gridDim.x;
   const long long t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
-  struct Tile {
-    int tm, tn, a, sp, b, bg, nst;
-    long long kc0;
-  };
-  auto tile_at = [&](long long t) {
-    Tile q;
-    q.tm = (int)(t % g.ntm);
-    t /= g.ntm;
-    q.tn = (int)(t % g.ntn);
-    const int z = (int)(t / g.ntn);
-    q.a = NN ? 0 : z % g.amod;
-    q.sp = NN ? 0 : z / g.amod;
-    q.b = NN ? z : 0;
-    q.bg = NN ? z % g.amod : 0;  // NN: amod holds bmod
-    q.kc0 = (long long)q.sp * g.kst * (kOzKT / 2);  // first complex k
-    q.nst = (int)min((long long)g.kst, (g.K - q.kc0 + kOzKT / 2 - 1) / (kOzKT / 2));
-    return q;
-  };
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
@@ -221,10 +384,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
     if (lane == 0) {
       const uint32_t idesc = (1u << 4)                        // D: F32; A, B: F16
                              | ((uint32_t)(128 >> 4) << 24);  // M >> 4; N >> 3 at bit 17
+      // magnitudes: A, B E5M2
+      const uint32_t sdesc = idesc | (1u << 7) | (1u << 10) | (ns >> 3) << 17;
       int u = 0;
       bool live = true;
       for (long long t = t0; t < t1 && live; ++t) {
-        const int nst = tile_at(t).nst;
+        const int nst = oz_tile<NN>(g, t).nst;
         for (int it = 0; it < nst; ++it, ++u) {
           const int s = u & 1;
           if (!mbar_wait(smem_u32(&full[s]), (uint32_t)((u >> 1) & 1))) {
@@ -259,6 +424,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
             }
           }
           asm volatile(
+              "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+              "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                  tmem + (uint32_t)(kOzS * nt) + ((t - t0) & 1 ? ns : 0u)),
+              "l"(smem_desc(ab + sOff, 2048, 128)),
+              "l"(smem_desc(ab + sOff + kOzSTile, ns * 16, 128)), "r"(sdesc), "r"((uint32_t)it));
+          asm volatile(
               "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                   smem_u32(&empty[s])));
         }
@@ -278,28 +449,21 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
     long long kc = 0;
     int nst = 0;
     auto operands = [&](long long t) {
-      const Tile q = tile_at(t);
+      const OzTile q = oz_tile<NN>(g, t);
       kc = q.kc0;
       nst = q.nst;
       rp = cp = nullptr;
       re = ce = 1;
-      const long long R = (long long)q.tm * 128 + rrow;
-      if (NN) {
-        if (R < g.ncol) {
-          rp = g.B + q.bg * g.sB + R;
-          re = g.eb[q.bg * g.ncol + R];
-        }
-      } else if (R < g.ntot) {
-        const int j = (int)(R / g.N), n = (int)(R - (long long)j * g.N);
-        const long long b = q.a + (long long)j * g.amod;
-        rp = g.B + b * g.sB + (long long)n * g.ldb;
-        re = g.eb[b * g.N + n];
+      const OzRow r = oz_row<NN>(g, q, (long long)q.tm * 128 + rrow);
+      if (r.in) {
+        rp = NN ? g.B + q.bg * g.sB + r.n : g.B + r.b * g.sB + r.n * g.ldb;
+        re = g.eb[r.e];
       }
       const int cg = q.tn * g.mt + cm;
       if (cm < g.mt && cg < g.M) {
         cp = NN ? g.A + q.b * g.sA + (long long)cg * g.sar
                 : g.A + q.a * g.sA + (long long)cg * g.lda;
-        ce = NN ? g.ea[(long long)q.b * g.M + cg] : g.ea[(long long)q.a * g.M + cg];
+        ce = g.ea[oz_col<NN>(g, q, cg)];
       }
     };
     // the thread's elements of a stage, copied a stage ahead: raw[u][thread], then the column
@@ -377,33 +541,71 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
     };
     // outputs of a tile: row 32 quarter + lane; columns (2m, 2m + 1) = (Re, Im); sums cleared
     auto output = [&](long long t) {
-      const Tile q = tile_at(t);
-      const long long R = (long long)q.tm * 128 + 32 * quarter + lane;
-      if (R < (NN ? g.ncol : (long long)g.ntot)) {
-        const int j = NN ? 0 : (int)(R / g.N), n = NN ? 0 : (int)(R - (long long)j * g.N);
-        const long long b = NN ? q.b : q.a + (long long)j * g.amod;
-        const int er = NN ? g.eb[q.bg * g.ncol + R] : g.eb[b * g.N + n];
-        const int m0 = q.tn * g.mt + cq * (nt >> 3);
-        const int nm = min(min(nt >> 3, g.mt - cq * (nt >> 3)), g.M - m0);
-        const int *ep = g.ea + (NN ? b : (long long)q.a) * g.M + m0;
-        const long long at = NN ? b * g.sO + (long long)m0 * g.ldo + R
-                                : (((long long)q.sp * g.batch + b) * g.M + m0) * g.N + n;
+      // sums of magnitudes (the next tile's are in the other half of their columns)
+      float mags[kOzMaxNt / 8];
+#pragma unroll
+      for (int i = 0; i < kOzMaxNt / 16; ++i) {
+        uint32_t r0 = 0, r1 = 0;
+        if (i < ngrp)
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];"
+                       : "=r"(r0), "=r"(r1)
+                       : "r"(tmem + ((uint32_t)(32 * quarter) << 16) + kOzS * nt +
+                             ((t - t0) & 1 ? ns : 0u) + (uint32_t)(cq * (nt >> 3) + 2 * i)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        mags[2 * i] = __uint_as_float(r0);
+        mags[2 * i + 1] = __uint_as_float(r1);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      const OzTile q = oz_tile<NN>(g, t);
+      const OzRow row = oz_row<NN>(g, q, (long long)q.tm * 128 + 32 * quarter + lane);
+      const int m0 = q.tn * g.mt + cq * (nt >> 3);
+      const int nm = min(min(nt >> 3, g.mt - cq * (nt >> 3)), g.M - m0);
+      const long long c0 = oz_col<NN>(g, q, m0);
+      const int er = row.in ? g.eb[row.e] : 1;
+      const int *ep = g.ea + c0;
+      uint32_t w = 0;  // bits c: the slices may cost column c more than FP64 rounding
+      if (row.in) {
+        const float lim = g.nb[row.e] + g.rk;
+#pragma unroll
+        for (int c = 0; c < kOzMaxNt / 8; ++c)
+          if (c < nm && mags[c] < 0x1p19f * (lim + g.na[c0 + c])) w |= 1u << c;  // 2^28 2^-9
+      }
+      if (__any_sync(0xffffffffu, w != 0)) {
+#pragma unroll
+        for (int c = 0; c < kOzMaxNt / 8; ++c)
+          if (w >> c & 1) {
+            bool fine = !oz_meet(g.bb + 2 * row.e, g.ba + 2 * (c0 + c));
+            if (NN && !fine) {
+              // an addend as large as the bound takes the error with its own rounding:
+              // |In / alpha| >= 2^x in units of the rows' scales, 2^(er - 1022) 2^(em - 1022)
+              const double2 iv = g.In[oz_at<NN>(g, q, row, m0 + c)];
+              const int x =
+                  max(oz_exp(iv.x), oz_exp(iv.y)) - oz_exp(g.alpha) - (er + ep[c]) + 2043;
+              const float a = __int_as_float(min(max(x + 127, 0), 254) << 23);
+              fine = a >= 0x1p-9f * (g.nb[row.e] + g.rk + g.na[c0 + c]);
+            }
+            if (fine) w &= ~(1u << c);
+          }
+      }
+      const bool redo = __any_sync(0xffffffffu, w != 0);
+      if (lane == 0) g.redo[t * 16 + warp] = redo;
+      if (row.in && !(NN && redo)) {
         const double sg = NN && (q.b % g.neg_mod) >= g.neg_from ? -1.0 : 1.0;
 #pragma unroll
         for (int c = 0; c < kOzMaxNt / 8; ++c)
           if (c < nm) {
             const int em = ep[c];
+            const long long at = oz_at<NN>(g, q, row, m0 + c);
             double2 v;
             v.x = oz_value(hi[2 * c], lo[2 * c], er + em - 2112);
             v.y = oz_value(hi[2 * c + 1], lo[2 * c + 1], er + em - 2112);
             if (er == 0x7ff || em == 0x7ff || !ok)  // non-finite operand, or expired wait
               v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
             if (NN) {
-              const double2 iv = g.In[at + (long long)c * g.ldo];
-              g.Out[at + (long long)c * g.ldo] =
-                  make_double2(sg * fma(g.alpha, v.x, iv.x), sg * fma(g.alpha, v.y, iv.y));
+              const double2 iv = g.In[at];
+              g.Out[at] = make_double2(sg * fma(g.alpha, v.x, iv.x), sg * fma(g.alpha, v.y, iv.y));
             } else {
-              g.part[at + (long long)c * g.N] = v;
+              g.part[at] = v;
             }
           }
       }
@@ -430,11 +632,18 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
           y[w] = oz_fix(v.y, re);
         }
         unsigned char *o = st + tile_off(rrow, rch, lboA);
+        uint4 lead;
 #pragma unroll
-        for (int d = 0; d < kOzS; ++d)
-          *reinterpret_cast<uint4 *>(o + d * kOzATile) =
-              make_uint4(oz_pair(x[0], y[0], 7 - d), oz_pair(x[1], y[1], 7 - d),
-                         oz_pair(x[2], y[2], 7 - d), oz_pair(x[3], y[3], 7 - d));
+        for (int d = 0; d < kOzS; ++d) {
+          const uint4 p = make_uint4(oz_pair(x[0], y[0], 7 - d), oz_pair(x[1], y[1], 7 - d),
+                                     oz_pair(x[2], y[2], 7 - d), oz_pair(x[3], y[3], 7 - d));
+          *reinterpret_cast<uint4 *>(o + d * kOzATile) = p;
+          if (d == 0) lead = p;
+          if (d == 1)
+            *reinterpret_cast<uint2 *>(st + sOff + tile_off(rrow, rch >> 1, 2048) +
+                                       8 * (rch & 1)) =
+                make_uint2(oz_mag(lead.x, p.x, lead.y, p.y), oz_mag(lead.z, p.z, lead.w, p.w));
+        }
         if (2 * cm < nt) {
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
@@ -445,11 +654,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
           unsigned char *oc = st + kOzS * kOzATile;
 #pragma unroll
           for (int d = 0; d < kOzS; ++d) {
-            uint32_t p[4], q[4];
+            uint32_t p[4], q[4], h4[4];
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
               // TN: Re row (x, y), Im row (-y, x); NN: Re row (x, -y), Im row (y, x)
               const uint32_t h = oz_pair(x[w], y[w], 7 - d), sw = __byte_perm(h, 0, 0x1032);
+              h4[w] = h;
               p[w] = NN ? h ^ 0x80000000u : h;
               q[w] = NN ? sw : sw ^ 0x00008000u;
             }
@@ -457,6 +667,16 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
                 make_uint4(p[0], p[1], p[2], p[3]);
             *reinterpret_cast<uint4 *>(oc + tile_off(d * nt + 2 * cm + 1, cc, lboB)) =
                 make_uint4(q[0], q[1], q[2], q[3]);
+            if (d == 0) lead = make_uint4(h4[0], h4[1], h4[2], h4[3]);
+            if (d == 1) {
+              // the larger of the two parts in both places: one sum for both parts of the output
+              uint2 m = make_uint2(oz_mag(lead.x, h4[0], lead.y, h4[1]),
+                                   oz_mag(lead.z, h4[2], lead.w, h4[3]));
+              m.x = __vmaxu4(m.x, __byte_perm(m.x, 0, 0x2301));
+              m.y = __vmaxu4(m.y, __byte_perm(m.y, 0, 0x2301));
+              *reinterpret_cast<uint2 *>(st + sOff + kOzSTile + tile_off(cm, cc >> 1, ns * 16) +
+                                         8 * (cc & 1)) = m;
+            }
           }
         }
         // this thread's elements of the next stage (its own slots: no barrier needed)
@@ -493,4 +713,64 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzArgs g) 
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
+
+// Blocks that oz_gemm_kernel left (32 rows x nt / 8 columns each) by FP64 multiply-adds: one row
+// per lane, the terms in runs of eight over the four warps (a row's run is one cache line), whose
+// sums are added in order.  A CTA looks through the flags of every gridDim.x-th quarter of a
+// tile's rows: nothing else to do for most calls (3 us).
+template <bool NN> __global__ void __launch_bounds__(128) oz_redo_kernel(const OzArgs g) {
+  constexpr int kC = kOzMaxNt / 8;
+  __shared__ double2 sh[4][kC][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  for (long long i = blockIdx.x; i < 4 * g.tiles; i += gridDim.x) {
+    const long long t = i >> 2;
+    const int quarter = (int)(i & 3);
+    const uint4 f = *reinterpret_cast<const uint4 *>(g.redo + t * 16);
+    if (((f.x | f.y | f.z | f.w) >> (8 * quarter) & 0xffu) == 0) continue;
+    const OzTile q = oz_tile<NN>(g, t);
+    const long long k1 = min(g.K, q.kc0 + (long long)q.nst * (kOzKT / 2));
+    for (int cq = 0; cq < 4; ++cq) {
+      if (!g.redo[t * 16 + 4 * cq + quarter]) continue;
+      const int m0 = q.tn * g.mt + cq * (g.nt >> 3);
+      const int nm = min(min(g.nt >> 3, g.mt - cq * (g.nt >> 3)), g.M - m0);
+      const OzRow row = oz_row<NN>(g, q, (long long)q.tm * 128 + 32 * quarter + lane);
+      double2 acc[kC];
+#pragma unroll
+      for (int c = 0; c < kC; ++c) acc[c] = make_double2(0.0, 0.0);
+      if (row.in) {
+        const double2 *bp = NN ? g.B + q.bg * g.sB + row.n : g.B + row.b * g.sB + row.n * g.ldb;
+        const double2 *ap = NN ? g.A + q.b * g.sA : g.A + q.a * g.sA;
+        for (long long kr = q.kc0 + 8 * part; kr < k1; kr += 32)
+          for (long long k = kr; k < min(k1, kr + 8); ++k) {
+            const double2 b = NN ? bp[k * g.ldb] : bp[k];
+#pragma unroll
+            for (int c = 0; c < kC; ++c)
+              if (c < nm) {
+                if (NN)
+                  cfma<double>(acc[c], __ldg(ap + (m0 + c) * g.sar + k * g.sak), b);
+                else
+                  cfmac<double>(acc[c], __ldg(ap + (m0 + c) * g.lda + k), b);
+              }
+          }
+      }
+#pragma unroll
+      for (int c = 0; c < kC; ++c) sh[part][c][lane] = acc[c];
+      __syncthreads();
+      for (int c = part; c < nm; c += 4)
+        if (row.in) {
+          double2 v = sh[0][c][lane];
+          for (int i = 1; i < 4; ++i) v = cadd<double>(v, sh[i][c][lane]);
+          const long long at = oz_at<NN>(g, q, row, m0 + c);
+          if (NN) {
+            const double2 iv = g.In[at];
+            const double2 h = mk<double>(fma(g.alpha, v.x, iv.x), fma(g.alpha, v.y, iv.y));
+            g.Out[at] = (q.b % g.neg_mod) >= g.neg_from ? mk<double>(-h.x, -h.y) : h;
+          } else {
+            g.part[at] = v;
+          }
+        }
+      __syncthreads();
+    }
+  }
 }
