@@ -138,9 +138,9 @@ struct QSlot {
   DevBuf pl_j1;   // [nk][nplane_max] grid index j1 of each plane
   DevBuf pl_of;   // [nk][n1] plane index of j1 or -1
   DevBuf st_id;   // [nk][nplane_max][n2] stick index of (plane, j2) or -1
-  // slab stages (slab.cu): planes of every k are one run of Miller indices m1 (grid indices
-  // 0 .. x-1 and the last y - x), stick -> plane (n2 + 1) + j2
-  bool slab_planes = false;
+  // slab stages (slab.cu): planes of every k within grid indices 0 .. x-1 and the last y - x
+  // (those without sticks are zeros), stick -> plane (n2 + 1) + j2
+  int slab_npm = 0;  // most planes of a k
   DevBuf slab_pl;   // [nk] int2 (planes from j1 = 0 up, planes in all)
   DevBuf slab_pos;  // [nk][nstick_max]
   // FP64 lines on the tensor cores (lines64.cuh), axes X and Y: largest |m1|, |m2| of the

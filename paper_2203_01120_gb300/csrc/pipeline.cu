@@ -998,20 +998,27 @@ void build_stick_tables(QSlot &s, const std::vector<int> &idx_kq) {
     end[0] = s.npw_kq[k];
   }
   s.st_runs = runs_ok;
-  // slab stages: stick positions in dense (plane, j2) rows of pitch n2 + 1, and each k's
-  // planes as a run from j1 = 0 up and a run that ends at n1 - 1
+  // slab stages: each k's planes within a run from j1 = 0 up and a run that ends at n1 - 1, the
+  // shortest that hold them (a sphere around zero fills them; one that a large q shifts away
+  // leaves planes without sticks, which are transformed as zeros), and stick positions in dense
+  // (plane, j2) rows of pitch n2 + 1
   std::vector<int> spos((size_t)nk * nsm, 0), spl((size_t)nk * 2, 0);
-  s.slab_planes = true;
+  s.slab_npm = 0;
   for (int k = 0; k < nk; ++k) {
-    int lo = 0;
-    while (lo < npl[k] && planes[k][lo] == lo) ++lo;
-    for (int p = lo; p < npl[k]; ++p)
-      if (planes[k][p] != n1 - npl[k] + p) s.slab_planes = false;
+    int lo = 0, all = n1 + 1;
+    for (int i = npl[k]; i >= 0; --i) {  // the first i planes in the lower run
+      const int a = i > 0 ? planes[k][i - 1] + 1 : 0, b = i < npl[k] ? n1 - planes[k][i] : 0;
+      if (a + b < all) {
+        lo = a;
+        all = a + b;
+      }
+    }
     spl[2 * k] = lo;
-    spl[2 * k + 1] = npl[k];
+    spl[2 * k + 1] = all;
+    s.slab_npm = std::max(s.slab_npm, all);
     for (int i = 0; i < nst[k]; ++i) {
-      const int c = sticks[k][i];
-      spos[(size_t)k * nsm + i] = plof[(size_t)k * n1 + c / n2] * (n2 + 1) + c % n2;
+      const int c = sticks[k][i], j1 = c / n2;
+      spos[(size_t)k * nsm + i] = (j1 < lo ? j1 : j1 - (n1 - all)) * (n2 + 1) + c % n2;
     }
   }
   auto up = [&](DevBuf &b, const std::vector<int> &v) {

@@ -488,7 +488,7 @@ SlabTab tab_of(const QSlot &s) {
   t.nb = s.nb;
   t.n3 = s.fft[2];
   t.nsm = s.nstick_max;
-  t.npm = s.nplane_max;
+  t.npm = s.slab_npm;
   t.gpp = (s.nb + nbs_of(s.fft[0]) - 1) / nbs_of(s.fft[0]);
   t.nnp = planes_nnp(s);
   return t;
@@ -513,15 +513,15 @@ int groups_of(const QSlot &s) {
 
 bool slab_supported(const QSlot &s) {
   const int n = s.fft[0];
-  if (s.fft[1] != n || !reg_fft_length(n) || !s.slab_planes) return false;
+  if (s.fft[1] != n || !reg_fft_length(n)) return false;
   size_t sm = kSlabSmem + 1;
   switch (n) {
-    case 12: sm = smem_inv<12>(s.nplane_max); break;
-    case 16: sm = smem_inv<16>(s.nplane_max); break;
-    case 24: sm = smem_inv<24>(s.nplane_max); break;
-    case 36: sm = smem_inv<36>(s.nplane_max); break;
-    case 45: sm = smem_inv<45>(s.nplane_max); break;
-    case 48: sm = smem_inv<48>(s.nplane_max); break;
+    case 12: sm = smem_inv<12>(s.slab_npm); break;
+    case 16: sm = smem_inv<16>(s.slab_npm); break;
+    case 24: sm = smem_inv<24>(s.slab_npm); break;
+    case 36: sm = smem_inv<36>(s.slab_npm); break;
+    case 45: sm = smem_inv<45>(s.slab_npm); break;
+    case 48: sm = smem_inv<48>(s.slab_npm); break;
     default: break;
   }
   return sm <= kSlabSmem && s.fft[2] <= 65535;
@@ -539,7 +539,7 @@ void slab_inverse_density(Context &ctx, QSlot &s, const float2 *i1t, const float
   const dim3 grid((unsigned)(nvec * nch), (unsigned)s.fft[2]);
 #define TDLZ_SLAB_INV(NV)                                                                     \
   {                                                                                           \
-    const size_t sm = smem_inv<NV>(s.nplane_max);                                             \
+    const size_t sm = smem_inv<NV>(s.slab_npm);                                             \
     auto kern = density ? slab_inverse_kernel<NV, true> : slab_inverse_kernel<NV, false>;     \
     TDLZ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
     kern<<<grid, Slab<NV>::ITH, sm, ctx.stream>>>(i1t, us, wk, xs, part, tab_of(s), nvec,  \

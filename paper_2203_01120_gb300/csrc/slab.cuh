@@ -6,7 +6,7 @@
 namespace tdlz {
 
 // True when slot s can run the slab stages: square x-y grid of a register-line length,
-// every k+q sphere's planes one run of Miller indices, shared memory within the limit.
+// shared memory within the limit.
 bool slab_supported(const QSlot &s);
 
 // Slices of the partial density (a function of the slot only: it fixes the summation order).
