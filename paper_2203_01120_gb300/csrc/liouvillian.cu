@@ -742,6 +742,14 @@ double staged_vector_bytes(const QSlot &s, size_t c) {
   return (double)s.rows() * per_row * (double)c;
 }
 
+// Bytes per stacked vector of the density slices, densities, potentials and Hartree grids beside
+// them (slab stages: up to a fifth of the grids with many k points on a flat cell, 48 x 48 x 12).
+double staged_field_bytes(const QSlot &s, size_t c) {
+  const bool slab = c == sizeof(float2) && s.slab32;
+  const double grids = slab ? 4.0 * slab_density_chunks(s) + 11.0 : 4.0 * kDensityGroups + 9.0;
+  return grids * (double)s.nr * (double)c;
+}
+
 // Stacked vectors the staged pipeline's buffers are sized for, decided when they are
 // allocated: all nvec where they take at most 70% of the memory then free (and at most
 // half the device), else the largest count that does (at least one).  The count
@@ -754,7 +762,7 @@ int staged_cap(const QSlot &s, size_t c, int nvec) {
     free_b = 0;
   }
   const double budget = std::min(0.5 * (double)s.dev_total, 0.7 * (double)free_b);
-  int n = (int)std::floor(budget / staged_vector_bytes(s, c));
+  int n = (int)std::floor(budget / (staged_vector_bytes(s, c) + staged_field_bytes(s, c)));
   n = std::max(1, std::min(n, nvec));
   if (s.staged_sub_env > 0) n = std::min(n, s.staged_sub_env);
   return n;
