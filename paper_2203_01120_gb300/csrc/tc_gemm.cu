@@ -1419,12 +1419,16 @@ bool tc_gemm_nn_img(Context &ctx, const TcImage &im, DevBuf &scratch, const floa
 namespace {
 
 // Clocks of `tiles` tiles of nst stages over the persistent CTAs (one per SM): the MMAs or the
-// operands' split per stage, a drain every four and at the end, the outputs.  Taken below 0.7
-// of the FP64-pipe form's clocks: at 24 x 24 x 48, 18 bands, 4 k points (V_NL 0.101 ms by the pipe,
-// 0.100 by slices, P_c 0.114 and 0.105) the two meet.
-double oz_clocks(double tiles, double nst, int nt) {
+// operands' split per stage, a drain every four and at the end, the outputs, and the launches
+// beside (rows' scales, blocks left to FP64 multiply-adds).  Taken below 0.7 of the FP64-pipe
+// form's clocks.  V_NL and P_c of one vector, 16^3 and 24 x 24 x 48 cells, 8 to 70 bands, 1 to 24 k
+// points, pipe -> rule: P_c 16^3, 25 bands, 4 k points 84 -> 84 us, 6 k points 137 -> 106; 70 bands, 2
+// k points V_NL 166 -> 110, P_c 297 -> 113; the worst, 24 x 24 x 48, 18 bands, 2 k points, P_c 87 ->
+// 99.  With 15000 clocks beside both, 11 of 86 such calls lost 7 to 16 us near the line.
+constexpr double kOzBesideTn = 27000.0, kOzBesideNn = 40000.0;
+double oz_clocks(double tiles, double nst, int nt, double beside) {
   const double tile = nst * 4500.0 + std::ceil(nst / kOzDrain) * 60.0 * nt + 4000.0;
-  return std::ceil(tiles / 152.0) * tile + 15000.0;
+  return std::ceil(tiles / 152.0) * tile + beside;
 }
 
 void oz_tiles(OzArgs &g) {
@@ -1521,7 +1525,7 @@ bool tc_gemm64_tn(Context &ctx, DevBuf &partbuf, const double2 *A, long long lda
     const long long st = ((nst + ns - 1) / ns + kOzDrain - 1) / kOzDrain * kOzDrain;
     const long long n = (nst + st - 1) / st;
     if (OzScratch(ra * n, rb * n, tiles * n).bytes + n * one > partbuf.bytes) break;
-    const double t = oz_clocks((double)tiles * n, (double)st, g.nt);
+    const double t = oz_clocks((double)tiles * n, (double)st, g.nt, kOzBesideTn);
     if (kst == 0 || t < best) {
       best = t;
       kst = st;
@@ -1583,7 +1587,7 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
   g.kst = (K + kOzKT / 2 - 1) / (kOzKT / 2);
   g.ntm = (int)oz_row_tiles(ncol);
   g.tiles = (long long)g.ntm * g.ntn * batch;
-  if (oz_clocks((double)g.tiles, (double)g.kst, g.nt) > 0.7 * clocks) return false;
+  if (oz_clocks((double)g.tiles, (double)g.kst, g.nt, kOzBesideNn) > 0.7 * clocks) return false;
   const long long ra = (long long)batch * rows, cb = (long long)bmod * ncol;
   const OzScratch sc(ra, cb, g.tiles);
   if (scratch.bytes < sc.bytes) return false;
@@ -1593,7 +1597,7 @@ bool tc_gemm64_nn(Context &ctx, DevBuf &scratch, const double2 *A, long long sA,
       A, rows, sA, sar, sak, K, K, const_cast<int *>(g.ea), const_cast<float *>(g.na),
       (uint32_t *)g.ba);
   TDLZ_LAUNCH_CHECK();
-  oz_col_scale_kernel<<<blocks_for(cb), 256, 0, ctx.stream>>>(
+  oz_col_scale_kernel<<<blocks_for(cb, 64), 64, 0, ctx.stream>>>(
       B, ldb, sB, bmod, K, ncol, const_cast<int *>(g.eb), const_cast<float *>(g.nb),
       (uint32_t *)g.bb);
   TDLZ_LAUNCH_CHECK();

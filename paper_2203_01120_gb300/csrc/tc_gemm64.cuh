@@ -216,7 +216,7 @@ __global__ void oz_col_scale_kernel(const double2 *__restrict__ B, long long ldb
     for (int w = 0; w < 4; ++w) {
       const int k0 = 128 * h + 32 * w;
       m[w] = 0;
-#pragma unroll 4
+#pragma unroll 16
       for (int k = k0; k < min(K, k0 + 32); ++k) {
         const double2 v = q[(long long)k * ldb];
         a.add(v);
