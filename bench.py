@@ -287,9 +287,10 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-# DRAM bytes per launch of a stage's kernel (dram__bytes_read.sum + dram__bytes_write.sum), for
-# the stages that have been captured at the benchmark's size.
-NCU_TRAFFIC = {}
+# DRAM bytes per launch of a stage's kernel (dram__bytes_read.sum + dram__bytes_write.sum), from an
+# ncu capture: slab_forward_kernel on six stacked vectors of C2's grid at 4 of the 16 k points,
+# scaled by 4 (its traffic is linear in the k points).  Summary: profiles/kernels_C2_k4.md.
+NCU_TRAFFIC = {("C2", "product"): 4 * 5.079e9}
 
 
 # GB300's FP64 vector rate (nominal, dense), the roof of the FP64 path's pointwise stages and Z

@@ -225,8 +225,8 @@ tdlz_status tdlz_lanczos_run(tdlz_ctx *ctx, const tdlz_lanczos_params *p, tdlz_l
 
 /* chi[nchain][ncomp][nomega] (complex double, caller-owned HOST array; ncomp = 3
  * or 4 as in tdlz_coeffs, so row l of chain c is chi_{l, mu_c}) for the
- * frequency grid of sp; FP64 on the GPU, one tridiagonal LU with partial
- * pivoting per (chain, omega).  *nomega receives the grid length; pass
+ * frequency grid of sp; FP64 on the GPU, one sweep of the tridiagonal's
+ * continuants per (chain, omega, row).  *nomega receives the grid length; pass
  * chi = NULL to query it. */
 tdlz_status tdlz_spectrum(tdlz_ctx *ctx, const tdlz_coeffs *c, const tdlz_spectrum_params *sp,
                           double *chi, int *nomega);

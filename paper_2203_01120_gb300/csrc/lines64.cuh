@@ -36,7 +36,8 @@ constexpr unsigned long long kLnBias = 0x0802008020080200ull;  // 512 (1 + 2^10 
 
 // fewest tiles of one vector that take this path (not of all the stacked ones: a group's result
 // is that of its sub-batches), four per CTA: 256 tiles of length 16 took 13.8 us where one thread
-// per line takes 11.6
+// per line takes 11.6.  The rule lies where slices meet the FP64 register lines (12, 16, 24, 36,
+// 45); other lengths run Stockham passes below it, not measured against slices of few tiles
 constexpr long long kLnMinTiles = 608;
 
 struct LineArgs {

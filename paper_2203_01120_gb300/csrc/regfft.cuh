@@ -45,7 +45,8 @@ __device__ __forceinline__ cx<T> rtw(const RegTw<T, N> &tw, int t) {
 // Complex sums, differences and real multiples s a + c of a line transform.  With PK
 // (FP32) both parts go through one packed instruction: the FP32 lanes do the same work in
 // half the issue slots, and half of a transform's instructions are these.
-// One vector of the 36 x 36 x 96 slab (16 k points), fused Y + X lines, inverse / forward:
+// One vector of the 36 x 36 x 96 slab (16 k points), Y + X lines in one kernel (the form before
+// the slab stages), inverse / forward:
 // Stockham stages 4-3-3 0.576 / 0.614 ms; this form scalar 0.593 / 0.627 ms (more registers,
 // one CTA less per SM), packed with the register budget of four CTAs 0.505 / 0.587 ms.
 // 45 x 45 x 144, four vectors, 8 k points: 6.38 / 6.23 -> 5.46 / 5.28 ms.  FP64 (bound by

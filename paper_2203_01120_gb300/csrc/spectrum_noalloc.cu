@@ -1,4 +1,4 @@
-// tdlz_spectrum_noalloc: the pivoted tridiagonal spectrum solve for callers that
+// tdlz_spectrum_noalloc: the tridiagonal spectrum solve (continuants) for callers that
 // cannot allocate device memory.  Inputs and outputs are the caller's device
 // buffers; the solve keeps its state in registers (spectrum_solve.cuh).
 #include <cmath>

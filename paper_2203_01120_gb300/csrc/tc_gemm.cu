@@ -1421,10 +1421,10 @@ namespace {
 // Clocks of `tiles` tiles of nst stages over the persistent CTAs (one per SM): the MMAs or the
 // operands' split per stage, a drain every four and at the end, the outputs, and the launches
 // beside (rows' scales, blocks left to FP64 multiply-adds).  Taken below 0.7 of the FP64-pipe
-// form's clocks.  V_NL and P_c of one vector, 16^3 and 24 x 24 x 48 cells, 8 to 70 bands, 1 to 24 k
-// points, pipe -> rule: P_c 16^3, 25 bands, 4 k points 84 -> 84 us, 6 k points 137 -> 106; 70 bands, 2
-// k points V_NL 166 -> 110, P_c 297 -> 113; the worst, 24 x 24 x 48, 18 bands, 2 k points, P_c 87 ->
-// 99.  With 15000 clocks beside both, 11 of 86 such calls lost 7 to 16 us near the line.
+// form's clocks.  V_NL and P_c of one vector, 16^3 and 24 x 24 x 48 cells, 8 to 70 bands, 1 to 24
+// k points, pipe -> rule: P_c 16^3, 25 bands, 4 k points 85 -> 84 us, 6 k points 137 -> 106; 70
+// bands, 2 k points V_NL 166 -> 111, P_c 298 -> 111; the worst, 24 x 24 x 48, 18 bands, 2 k points,
+// P_c 86 -> 99.  With 15000 clocks beside both, 11 of 86 such calls lost 7 to 16 us near the line.
 constexpr double kOzBesideTn = 27000.0, kOzBesideNn = 40000.0;
 double oz_clocks(double tiles, double nst, int nt, double beside) {
   const double tile = nst * 4500.0 + std::ceil(nst / kOzDrain) * 60.0 * nt + 4000.0;

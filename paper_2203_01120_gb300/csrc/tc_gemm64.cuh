@@ -38,11 +38,12 @@
 // multiplied by its 8 - i column digits side by side in one or two MMAs, so that it is read
 // twice at most (one MMA per pair: 7% more time).  Tiles follow
 // each other without a refill of the stages: with one CTA per tile the update's three stages
-// paid start and drain each time (V_NL and P_c of 0.52 and 0.67 ms for 0.38 and 0.41 below).
+// paid start and drain each time (V_NL and P_c of 0.52 and 0.67 ms for 0.38 and 0.41).
 // Bound by the split's integer instructions beside the MMAs.  Measured, FP64 pipe -> slices,
-// one vector: 36 x 36 x 96 grid, 40 bands, 4 k points: V_NL 3.17 -> 0.51 ms, P_c 2.16 -> 0.57;
-// 45 x 45 x 144, 24 bands, 2 k points: V_NL 2.25 -> 0.36, P_c 0.93 -> 0.39.  Relative error of
-// L x against 64-bit sums: 1.298e-16 -> 1.278e-16 and 4.104e-16 -> 4.101e-16.
+// one vector: 36 x 36 x 96 grid, 40 bands, 4 k points: V_NL 3.17 -> 0.55 ms, P_c 2.16 -> 0.57 (of
+// that the rows' scales 0.07 and 0.06, the second kernels 0.01 each); 45 x 45 x 144, 24 bands, 2 k
+// points: V_NL 2.25 -> 0.35, P_c 0.93 -> 0.33.  Relative error of L x against 64-bit sums:
+// 1.298e-16 -> 1.284e-16 and 4.104e-16 -> 4.104e-16.
 #pragma once
 
 constexpr int kOzS = 8;                       // digits
